@@ -1,22 +1,31 @@
 // fastbuild.cu -- bucketed construction: ArrayFill in shared memory.
 //
-// The keys of a level are kept grouped by position range ("buckets" of P
-// consecutive positions of A_d, P a power of two).  One CTA then runs the
-// whole of Algorithm 2 for a bucket with its hit / collision bits in shared
-// memory (no L2 atomics), writes the bucket's slice of A_d with plain stores
-// and counts weight(A_d).  Once every bucket is filled, |F_{d+1}| =
-// |F_d| - weight(A_d) and |A_{d+1}| are known, so compaction can place each
-// surviving key straight into its level-(d+1) bucket: the survivors of a tile
-// are counting-sorted by destination bucket in shared memory, one atomicAdd
-// per (tile, bucket) reserves their slots, and they are written out as
-// contiguous runs.  The caller's keys are first partitioned the same way for
-// level 0.  Levels with at most T keys run in a single CTA (k_tail) that keeps
-// keys and bit arrays in shared memory and loops over all remaining levels,
-// sorting the fallback (Sec. 3.5) at the end.
+// A level runs in two launches.  k_split hashes the level's keys and writes
+// them to position buckets (P consecutive positions of A_d, P a power of two)
+// through the write-combining multisplit of split.cuh.  k_fill_compact then
+// runs Algorithm 2 for a bucket with its hit / collision bits in shared memory
+// (no L2 atomics), writes the bucket's slice of A_d, and appends the keys whose
+// bit is 0 to F_{d+1}.  Once every bucket is done |F_{d+1}| and |A_{d+1}| are
+// known and level d+1's split can run.  Levels with at most T keys run in a
+// single CTA (k_tail) that keeps keys and bit arrays in shared memory and loops
+// over all remaining levels, sorting the fallback (Sec. 3.5) at the end.
 //
-// Every bound (bucket capacity, bucket count, flat buffer) is checked on the
-// device; when one is exceeded the build is redone by the unbucketed path in
-// build.cu, so results never depend on these choices.
+// Buckets and F hold h_d(x), not x: the hash is a bijection of 64-bit values
+// (unmix64), so its value stands for the key, the position costs one multiply
+// instead of a stored 4-byte position or a second hash, and only the survivors
+// of a level are hashed again.  A visit of a key reads and writes 8 bytes in
+// the split, reads 8 twice in the fill (the second time partly from L2) and
+// writes 8 per survivor.
+//
+// Every bound (bucket capacity, bucket count, F) is checked on the device;
+// when one is exceeded the build is redone by the unbucketed path in build.cu,
+// so results never depend on these choices.
+//
+// Measured (GB300, 1e8 keys, gamma = 2, 763 buckets at level 0): split of
+// level 0 0.43 ms, of all levels 0.88 ms; fill and compaction 0.38 / 0.76 ms;
+// build 1.79 ms.  A counting-sort multisplit that stored (key, position) pairs,
+// with a fill and a compaction that fed the next level's multisplit, took 0.89
+// ms for level 0, 0.32 + 1.02 ms for fills and compactions, 2.34 ms in all.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdlib.h>
@@ -24,84 +33,38 @@
 
 #include "fastbuild.cuh"
 #include "sector.cuh"
+#include "split.cuh"
 
 namespace bbh {
 
 
-// Each thread owns kKPT consecutive keys of a tile, staged by asynchronous
-// copies: a thread takes its keys of tile t into registers, then starts
-// copying its keys of the next tile into the same slots while tile t is
-// split.  Slot layout: pair q (keys 2q, 2q+1) of thread t at 16-byte unit
-// q * kTT + t, so a warp's reads of one pair hit consecutive 16-byte units.
-template <bool ALIGNED>
-__global__ void __launch_bounds__(kTT, 2)
-k_partition0(const u64 *__restrict__ keys, u64 n, FastMeta *__restrict__ meta, FastCfg cfg) {
+// Split of level d: the caller's keys (d = 0) or the survivors of level d - 1
+// (F, as values h_{d-1}) to the position buckets of A_d, as values h_d.
+template <int OWN, bool FIRST>
+__global__ void __launch_bounds__(kWT, 1)
+k_split(const u64 *__restrict__ keys, u64 n, FastMeta *__restrict__ meta, int d, FastCfg cfg,
+        unsigned nb_max) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const FLevel lv = meta->lv[0];
-  const unsigned nb = (unsigned)lv.B;
-  SplitSmem sm = carve_split(smem, (unsigned)kBmax);
-  split_clear(sm, nb);
-  __syncthreads();
-  u64 *inbuf = reinterpret_cast<u64 *>(smem + split_smem_bytes((unsigned)kBmax));
-  auto slot = [&](int k) -> u64 * { return inbuf + 2 * ((k >> 1) * kTT + threadIdx.x) + (k & 1); };
-  const u64 s0 = level_seed(cfg.seed, 0);
-  const unsigned sh = ilog2_u64(lv.P);
-  const unsigned mask = (unsigned)(lv.P - 1);
-  const u64 ntiles = ceil_div(n, kTile);
-  const unsigned base = threadIdx.x * kKPT;
-  auto prefetch = [&](u64 t) {
-    if (t < ntiles) {
-      const u64 *src = keys + t * kTile;
-      const u64 rem = n - t * kTile;
-      const unsigned nt = rem < (u64)kTile ? (unsigned)rem : (unsigned)kTile;
-      if (ALIGNED && base + kKPT <= nt) {
-#pragma unroll
-        for (int k = 0; k < kKPT; k += 2) cp_async16(slot(k), src + base + k);
-      } else {
-#pragma unroll
-        for (int k = 0; k < kKPT; k++)
-          if (base + k < nt) cp_async8(slot(k), src + base + k);
-      }
-    }
-    cp_async_commit();
-  };
-  u64 t = blockIdx.x;
-  prefetch(t);
-  for (; t < ntiles; t += gridDim.x) {
-    cp_async_wait0();  // this thread's copies of tile t have landed
-    const u64 rem = n - t * kTile;
-    const unsigned nt = rem < (u64)kTile ? (unsigned)rem : (unsigned)kTile;
-    u64 x[kKPT];
-    bool ok[kKPT];
-#pragma unroll
-    for (int k = 0; k < kKPT; k += 2) {
-      const uint4 v = *reinterpret_cast<const uint4 *>(slot(k));
-      x[k] = ((u64)v.y << 32) | v.x;
-      x[k + 1] = ((u64)v.w << 32) | v.z;
-    }
-#pragma unroll
-    for (int k = 0; k < kKPT; k++) {
-      ok[k] = base + k < nt;
-      if (!ok[k]) x[k] = 0;
-    }
-    prefetch(t + gridDim.x);
-    unsigned dst[kKPT], lp[kKPT];
-#pragma unroll
-    for (int k = 0; k < kKPT; k++) {
-      const u64 p = ok[k] ? level_pos(x[k], s0, lv.m) : 0;
-      dst[k] = (unsigned)(p >> sh);
-      lp[k] = (unsigned)p & mask;
-    }
-    multisplit_write<true>(x, lp, dst, ok, nb, sm, cfg.X, cfg.XP, UniformDest{cfg.cntX, lv.cap},
-                           &meta->status);
+  // one decision for the whole CTA: another CTA may be raising the status now
+  if (__syncthreads_or(meta->lv[d].mode != LM_BUCKETED || *(volatile unsigned *)&meta->status))
+    return;
+  const FLevel lv = meta->lv[d];
+  if (lv.B > nb_max) {  // more buckets than the rings were sized for
+    if (threadIdx.x == 0) atomicOr(&meta->status, ST_OVERFLOW);
+    return;
   }
-  cp_async_wait0();
+  const WcShape sh = wc_shape((unsigned)lv.B);
+  const u64 s_d = level_seed(cfg.seed, d);
+  const u64 s_x = FIRST ? s_d : s_d ^ level_seed(cfg.seed, d - 1);
+  const unsigned m = (unsigned)lv.m, shift = ilog2_u64(lv.P);
+  wc_split<OWN>(
+      FIRST ? keys : cfg.F, FIRST ? n : lv.n, sh, smem,
+      [=](u64 v) { return mix64((FIRST ? v : unmix64(v)) ^ s_x); },
+      [=](u64 y) { return reduce_range32(y, m) >> shift; }, UniformDest{cfg.cnt, lv.cap}, cfg.X,
+      &meta->status);
 }
 
-// ---------------------------------------------------------------------------
-// Fill (Algorithm 2) of level d, one bucket per CTA iteration, bits in shared
-// memory; writes A_d and weight(A_d); the last CTA sizes level d+1.
-// ---------------------------------------------------------------------------
+// |F_{d+1}| = |F_d| - weight(A_d); level d+1's size and where it lives.
 __device__ void finish_level(FastMeta *meta, int d, const FastCfg &cfg) {
   volatile FLevel *vl = meta->lv;
   const u64 n = vl[d].n, m = vl[d].m, w = vl[d].weight;
@@ -116,7 +79,6 @@ __device__ void finish_level(FastMeta *meta, int d, const FastCfg &cfg) {
     meta->levels_used = d + 1;
   } else if ((uint32_t)(d + 1) == cfg.L) {
     nx.mode = LM_FLAT;  // fallback
-    if (nn > cfg.flat_cap) atomicOr(&meta->status, ST_OVERFLOW);
   } else if (nn <= cfg.T) {
     nx.mode = LM_FLAT;  // tail
     nx.m = level_bits(nn, cfg.gamma);
@@ -124,11 +86,10 @@ __device__ void finish_level(FastMeta *meta, int d, const FastCfg &cfg) {
     size_bucketed(nx, nn, cfg.gamma, cfg.Pmin, cfg.Pmax, cfg.Btarget, cfg.cap_scale);
     nx.off = vl[d].off + m;
     nx.mode = LM_BUCKETED;
-    // the arenas were allocated before level 0 ran (level 1's from a bound on
-    // |F_1|): a level that does not fit sends the build to the unbucketed path
-    const u64 acap = ((d + 1) & 1) ? cfg.capY : cfg.capX;
+    // the arena was allocated before level 0 ran (from a bound on |F_1|): a
+    // level that does not fit sends the build to the unbucketed path
     const bool a_fits = ((nx.off - cfg.m0) >> 6) + (nx.m >> 6) <= cfg.arena_words;
-    if (nx.B > cfg.Bmax || nx.B * nx.cap > acap || !a_fits) {
+    if (nx.B > cfg.Bmax || nx.B * nx.cap > cfg.capX || !a_fits) {
       atomicOr(&meta->status, ST_OVERFLOW);
       nx.mode = LM_NONE;
     }
@@ -137,73 +98,157 @@ __device__ void finish_level(FastMeta *meta, int d, const FastCfg &cfg) {
   __threadfence();
 }
 
+// ---------------------------------------------------------------------------
+// ArrayFill (Algorithm 2) and compaction (Algorithm 1) of level d, one bucket
+// per CTA iteration with its hit and collision bits in shared memory.  Pass 1
+// streams the bucket's values and sets the bits; A_d's words of the bucket
+// leave and their ones are counted, which also fixes the number of survivors
+// (values in the bucket less ones), so one global atomic reserves the whole
+// bucket's run of F_{d+1}.  Pass 2 streams the values again and writes those
+// whose bit is 0, each warp taking its part of the run with a shared-memory
+// atomic.  The last CTA sizes level d+1.
+// ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kTT, 2)
-k_fill_buckets(FastMeta *__restrict__ meta, int d, FastCfg cfg) {
+k_fill_compact(FastMeta *__restrict__ meta, int d, FastCfg cfg) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ u64 red[kTT / 32];
-  __shared__ unsigned sred[kTT / 32 + 2];
+  __shared__ u64 s_base;
+  __shared__ unsigned s_count, s_room;
   __shared__ bool last;
-  if (meta->lv[d].mode != LM_BUCKETED || meta->status) return;
+  if (__syncthreads_or(meta->lv[d].mode != LM_BUCKETED || *(volatile unsigned *)&meta->status))
+    return;
   const FLevel lv = meta->lv[d];
-  const unsigned *parena = (d & 1) ? cfg.YP : cfg.XP;
-  const u64 *cnt = (d & 1) ? cfg.cntY : cfg.cntX;
   u64 *Alev = (d == 0) ? cfg.A0 : cfg.arena + ((lv.off - cfg.m0) >> 6);
   const unsigned Pw = (unsigned)(lv.P >> 5);  // 32-bit words per bit array
   unsigned *hit = reinterpret_cast<unsigned *>(smem);
   unsigned *col = hit + Pw;
-  u64 wsum = 0, got = 0;
+  const unsigned m = (unsigned)lv.m;
+  const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
+  u64 wtot = 0, got = 0;  // thread 0: ones and values of this CTA's buckets
   for (u64 b = blockIdx.x; b < lv.B; b += gridDim.x) {
-    for (unsigned i = threadIdx.x; i < 2 * Pw; i += kTT) hit[i] = 0;
+    for (unsigned i = threadIdx.x; i < Pw / 2; i += kTT)
+      reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0, 0, 0, 0);
+    const unsigned nk = (unsigned)min(cfg.cnt[b], lv.cap);
+    const u64 *yb = cfg.X + b * lv.cap;
+    const uint4 *y4 = reinterpret_cast<const uint4 *>(yb);  // cap % 16 == 0
+    const unsigned p0 = (unsigned)(b * lv.P);
+    const unsigned nv = nk >> 1;  // pairs of values
+    auto val0 = [](const uint4 &v) { return ((u64)v.y << 32) | v.x; };
+    auto val1 = [](const uint4 &v) { return ((u64)v.w << 32) | v.z; };
     __syncthreads();
-    const u64 nk = min(cnt[b], lv.cap);
-    got += (threadIdx.x == 0) ? cnt[b] : 0;
-    const unsigned *pb = parena + b * lv.cap;
-    const uint4 *pb4 = reinterpret_cast<const uint4 *>(pb);  // cap % 4 == 0: 16-byte aligned
-    // 4 positions per 16-byte load, U loads in flight per thread
+    // pass 1: U pairs in flight per thread
     constexpr int U = 4;
-    for (u64 i0 = threadIdx.x; 4 * i0 < nk; i0 += (u64)U * kTT) {
-      unsigned q[4 * U];
+    constexpr unsigned kStep = U * kTT;
+    const unsigned nsteps = (nv + kStep - 1) / kStep;
+    // step s of the bucket into L2 (its loads come later)
+    auto ahead = [&](unsigned s) {
+      if (threadIdx.x == 0 && s < nsteps)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(y4 + s * kStep),
+                     "r"(min(kStep, nv - s * kStep) * 16));
+    };
+    auto set = [&](u64 y) {
+      const unsigned q = reduce_range32(y, m) - p0;
+      const unsigned bit = 1u << (q & 31);
+      const unsigned old = atomicOr(hit + (q >> 5), bit);
+      if (old & bit) atomicOr(col + (q >> 5), bit);
+    };
+    ahead(1);
+    for (unsigned st = 0; st < nsteps; st++) {
+      const unsigned i0 = st * kStep + threadIdx.x;
+      ahead(st + 2);
+      uint4 v[U];
 #pragma unroll
       for (int u = 0; u < U; u++) {
-        const u64 i = i0 + (u64)u * kTT;
-        if (4 * i + 3 < nk) {
-          const uint4 v = __ldcs(pb4 + i);
-          q[4 * u] = v.x;
-          q[4 * u + 1] = v.y;
-          q[4 * u + 2] = v.z;
-          q[4 * u + 3] = v.w;
-        } else {
-#pragma unroll
-          for (int j = 0; j < 4; j++) q[4 * u + j] = (4 * i + j < nk) ? __ldcs(pb + 4 * i + j) : ~0u;
-        }
+        const unsigned i = i0 + (unsigned)u * kTT;
+        if (i < nv) v[u] = __ldcg(y4 + i);
       }
 #pragma unroll
-      for (int j = 0; j < 4 * U; j++) {
-        const unsigned p = q[j];
-        if (p != ~0u) {
-          const unsigned bit = 1u << (p & 31);
-          const unsigned old = atomicOr(hit + (p >> 5), bit);
-          if (old & bit) atomicOr(col + (p >> 5), bit);
+      for (int u = 0; u < U; u++) {
+        if (i0 + (unsigned)u * kTT < nv) {
+          set(val0(v[u]));
+          set(val1(v[u]));
         }
       }
     }
+    if ((nk & 1) && threadIdx.x == 0) set(yb[nk - 1]);
     __syncthreads();
-    // A_d words of this bucket: positions [b P, min((b+1) P, m))
+    // A_d words of this bucket: positions [b P, min((b+1) P, m)); hit keeps A
     const u64 w0 = (b * lv.P) >> 6;
-    const u64 wend = min((b + 1) * lv.P, lv.m) >> 6;
-    for (u64 w = w0 + threadIdx.x; w < wend; w += kTT) {
-      const unsigned j = (unsigned)(w - w0) * 2;
-      const u64 a = (u64)(hit[j] & ~col[j]) | ((u64)(hit[j + 1] & ~col[j + 1]) << 32);
-      Alev[w] = a;
-      wsum += __popcll(a);
+    const unsigned nw = (unsigned)((min((b + 1) * lv.P, lv.m) >> 6) - w0);
+    unsigned wsum = 0;
+    for (unsigned w = threadIdx.x; w < nw; w += kTT) {
+      const uint2 h2 = reinterpret_cast<uint2 *>(hit)[w], c2 = reinterpret_cast<uint2 *>(col)[w];
+      const uint2 a = make_uint2(h2.x & ~c2.x, h2.y & ~c2.y);
+      reinterpret_cast<uint2 *>(hit)[w] = a;
+      Alev[w0 + w] = ((u64)a.y << 32) | a.x;
+      wsum += __popc(a.x) + __popc(a.y);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) wsum += __shfl_down_sync(0xffffffffu, wsum, o);
+    if (lane == 0) red[threadIdx.x >> 5] = wsum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      u64 w = 0;
+      for (int i = 0; i < kTT / 32; i++) w += red[i];
+      wtot += w;
+      got += cfg.cnt[b];
+      const u64 ns = w > nk ? 0 : nk - w;
+      const u64 at = ns ? atomicAdd(&meta->n_out[d], ns) : 0;
+      const bool fits = w <= nk && at + ns <= cfg.F_cap;
+      if (!fits) atomicOr(&meta->status, ST_OVERFLOW);
+      s_base = at;
+      s_room = fits ? (unsigned)ns : 0u;
+      s_count = 0;
+    }
+    __syncthreads();
+    u64 *out = cfg.F + s_base;
+    const unsigned room = s_room;
+    // pass 2, last step first (it is the likeliest to be still in L2): a warp
+    // step takes U groups of 32 pairs
+    auto kept = [&](u64 y) {
+      const unsigned q = reduce_range32(y, m) - p0;
+      return !((hit[q >> 5] >> (q & 31)) & 1u);
+    };
+    for (unsigned st = nsteps; st-- > 0;) {
+      const unsigned i0 = st * kStep + threadIdx.x;
+      ahead(st - 2);
+      uint4 v[U];
+#pragma unroll
+      for (int u = 0; u < U; u++) {
+        const unsigned i = i0 + (unsigned)u * kTT;
+        v[u] = i < nv ? __ldcs(y4 + i) : make_uint4(0, 0, 0, 0);
+      }
+      unsigned bal[2 * U], tot = 0, keep = 0;
+#pragma unroll
+      for (int u = 0; u < U; u++) {
+        const bool ok = i0 + (unsigned)u * kTT < nv;
+        const bool k0 = ok && kept(val0(v[u])), k1 = ok && kept(val1(v[u]));
+        keep |= (k0 ? 1u : 0u) << (2 * u) | (k1 ? 1u : 0u) << (2 * u + 1);
+        bal[2 * u] = __ballot_sync(0xffffffffu, k0);
+        bal[2 * u + 1] = __ballot_sync(0xffffffffu, k1);
+        tot += __popc(bal[2 * u]) + __popc(bal[2 * u + 1]);
+      }
+      unsigned at = 0;
+      if (lane == 0 && tot) at = atomicAdd(&s_count, tot);
+      at = __shfl_sync(0xffffffffu, at, 0);
+      if (at + tot > room) continue;  // F_{d+1} is full (status raised)
+#pragma unroll
+      for (int u = 0; u < U; u++) {
+        if ((keep >> (2 * u)) & 1u) out[at + __popc(bal[2 * u] & lt)] = val0(v[u]);
+        at += __popc(bal[2 * u]);
+        if ((keep >> (2 * u + 1)) & 1u) out[at + __popc(bal[2 * u + 1] & lt)] = val1(v[u]);
+        at += __popc(bal[2 * u + 1]);
+      }
+    }
+    if ((nk & 1) && threadIdx.x == 0 && kept(yb[nk - 1])) {
+      const unsigned at = atomicAdd(&s_count, 1u);
+      if (at < room) out[at] = yb[nk - 1];
     }
     __syncthreads();
   }
-  const u64 tw = block_sum<kTT>(wsum, red);
-  const u64 tg = block_sum<kTT>(got, red);
   if (threadIdx.x == 0) {
-    if (tw) atomicAdd(&meta->lv[d].weight, tw);
-    if (tg) atomicAdd(&meta->seen[d], tg);
+    if (wtot) atomicAdd(&meta->lv[d].weight, wtot);
+    if (got) atomicAdd(&meta->seen[d], got);
     __threadfence();
     unsigned t = atomicAdd(&meta->lv[d].done, 1u);
     last = (t == gridDim.x - 1);
@@ -217,209 +262,18 @@ k_fill_buckets(FastMeta *__restrict__ meta, int d, FastCfg cfg) {
   }
   if (last) {
     __syncthreads();
-    // zero the counters of the arena that level d+1 is written into
+    // zero the bucket counters for level d+1's split
     const FLevel nx = meta->lv[d + 1];
-    if (nx.mode == LM_BUCKETED) {
-      u64 *c2 = ((d + 1) & 1) ? cfg.cntY : cfg.cntX;
-      for (u64 i = threadIdx.x; i < nx.B; i += kTT) c2[i] = 0;
-    }
-    // compaction units (kIn entries) before each bucket of level d, so that
-    // the compaction can hand every CTA the same number of units
-    const unsigned B = (unsigned)lv.B;
-    const unsigned per = (B + kTT - 1) / kTT;
-    const unsigned lo = threadIdx.x * per;
-    const unsigned hi = lo + per < B ? lo + per : B;
-    auto units = [&](unsigned b) -> unsigned {
-      const u64 nk = min(cnt[b], lv.cap);
-      return (unsigned)((nk + kIn - 1) / kIn);
-    };
-    unsigned su = 0;
-    for (unsigned b = lo; b < hi; b++) su += units(b);
-    unsigned total;
-    unsigned pre = block_scan_u32<kTT>(su, sred, &total);
-    for (unsigned b = lo; b < hi; b++) {
-      cfg.upre[b] = pre;
-      pre += units(b);
-    }
-    if (threadIdx.x == 0) cfg.upre[B] = total;
+    if (nx.mode == LM_BUCKETED)
+      for (u64 i = threadIdx.x; i < nx.B; i += kTT) cfg.cnt[i] = 0;
   }
 }
 
-// ---------------------------------------------------------------------------
-// Compaction of level d: keys whose A_d bit is 0 go to their level-(d+1)
-// bucket (or, for a small or final level, to the flat buffer).  The survivors
-// of a tile are first packed densely in shared memory so that their
-// level-(d+1) hashes are computed by full warps.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kTT, 2)
-k_compact_buckets(FastMeta *__restrict__ meta, int d, FastCfg cfg) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ unsigned scnt[3];  // survivors of the last three units (rotating)
-  if (meta->lv[d].mode != LM_BUCKETED || meta->status) return;
-  const FLevel lv = meta->lv[d];
-  const FLevel nx = meta->lv[d + 1];
-  if (nx.mode == LM_DONE || nx.mode == LM_NONE) return;
-  // this CTA's share of the level's units (kIn-entry slices of the buckets)
-  const unsigned *upre = cfg.upre;
-  const unsigned U = upre[lv.B];
-  const unsigned u0 = (unsigned)(((u64)U * blockIdx.x) / gridDim.x);
-  const unsigned u1 = (unsigned)(((u64)U * (blockIdx.x + 1)) / gridDim.x);
-  if (u0 >= u1) return;
-  const bool flat = nx.mode == LM_FLAT;
-  const unsigned nb = flat ? 1u : (unsigned)nx.B;
-  if (nb > cfg.nbcap) {  // more destinations than the arrays were sized for
-    if (threadIdx.x == 0) atomicOr(&meta->status, ST_OVERFLOW);
-    return;
-  }
-  // the stage holds up to kTile + kIn survivors: a full tile goes to the
-  // multisplit, the rest waits for the next one
-  SplitSmem sm = carve_split(smem, (unsigned)cfg.nbcap, kTile + kIn);
-  u64 *segA = reinterpret_cast<u64 *>(smem + split_smem_bytes((unsigned)cfg.nbcap, kTile + kIn));
-  u64 *stage = sm.sorted;
-  const u64 *arena = (d & 1) ? cfg.Y : cfg.X;
-  const unsigned *parena = (d & 1) ? cfg.YP : cfg.XP;
-  const u64 *cnt = (d & 1) ? cfg.cntY : cfg.cntX;
-  u64 *out = flat ? cfg.flat : (((d + 1) & 1) ? cfg.Y : cfg.X);
-  unsigned *pout = flat ? nullptr : (((d + 1) & 1) ? cfg.YP : cfg.XP);
-  u64 *ocnt = flat ? &meta->n_flat : (((d + 1) & 1) ? cfg.cntY : cfg.cntX);
-  const u64 ocap = flat ? cfg.flat_cap : nx.cap;
-  const u64 *Alev = (d == 0) ? cfg.A0 : cfg.arena + ((lv.off - cfg.m0) >> 6);
-  const u64 s_n = level_seed(cfg.seed, d + 1);
-  const unsigned shn = flat ? 0u : ilog2_u64(nx.P);
-  const unsigned maskn = flat ? 0u : (unsigned)(nx.P - 1);
-  const unsigned lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-
-  // bucket of unit u0: the last b with upre[b] <= u0 (empty buckets own no unit)
-  unsigned b = 0;
-  {
-    unsigned lo = 0, hi = (unsigned)lv.B;
-    while (hi - lo > 1) {
-      const unsigned mid = (lo + hi) >> 1;
-      if (upre[mid] <= u0) lo = mid;
-      else hi = mid;
-    }
-    b = lo;
-  }
-  unsigned ubase = upre[b], bnext = upre[b + 1];
-  auto load_segA = [&](unsigned bb) {
-    const u64 w0 = ((u64)bb * lv.P) >> 6;
-    const u64 wend = min((u64)(bb + 1) * lv.P, lv.m) >> 6;
-    for (u64 w = w0 + threadIdx.x; w < wend; w += kTT) segA[w - w0] = Alev[w];
-  };
-  if (threadIdx.x < 3) scnt[threadIdx.x] = 0;
-  split_clear(sm, nb);
-  load_segA(b);
-  __syncthreads();
-
-  // multisplit the ns staged survivors into level d+1's buckets (or the flat list)
-  auto flush = [&](unsigned ns) {
-    u64 x[kKPT];
-    unsigned dst[kKPT], lp[kKPT];
-    bool ok[kKPT];
-#pragma unroll
-    for (int k = 0; k < kKPT; k++) {
-      const unsigned i = (unsigned)k * kTT + threadIdx.x;
-      ok[k] = i < ns;
-      x[k] = ok[k] ? stage[i] : 0;
-      dst[k] = 0;
-      lp[k] = 0;
-      if (ok[k] && !flat) {
-        const u64 p = level_pos(x[k], s_n, nx.m);
-        dst[k] = (unsigned)(p >> shn);
-        lp[k] = (unsigned)p & maskn;
-      }
-    }
-    __syncthreads();  // the staging area is reused by the writer
-    if (flat)
-      multisplit_write<false>(x, lp, dst, ok, nb, sm, out, pout, UniformDest{ocnt, ocap},
-                              &meta->status);
-    else
-      multisplit_write<true>(x, lp, dst, ok, nb, sm, out, pout, UniformDest{ocnt, ocap},
-                             &meta->status);
-  };
-
-  unsigned ns = 0;  // staged survivors (the same value in every thread)
-  unsigned it = 0;
-  for (unsigned u = u0; u < u1; u++, it++) {
-    if (u >= bnext) {  // next non-empty bucket: its slice of A_d replaces the old one
-      do {
-        b++;
-        ubase = bnext;
-        bnext = upre[b + 1];
-      } while (u >= bnext);
-      __syncthreads();
-      load_segA(b);
-      __syncthreads();
-    }
-    // 1. test kInPT consecutive entries per thread (16-byte loads); a key whose
-    // A_d bit is 0 survives to F_{d+1} (Algorithm 1)
-    const u64 nk = min(cnt[b], lv.cap);
-    const u64 e0 = (u64)(u - ubase) * kIn + (u64)threadIdx.x * kInPT;
-    const unsigned *pe = parena + (u64)b * lv.cap + e0;
-    const u64 *ke = arena + (u64)b * lv.cap + e0;
-    // pull this thread's entries of the next unit of the bucket into L2 now, so
-    // that their loads one unit later do not wait for HBM
-    if (u + 1 < u1 && u + 1 < bnext && e0 + kIn < nk) {
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(ke + kIn));
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(pe + kIn));
-    }
-    unsigned pk[kInPT];
-    u64 xk[kInPT];
-    if (e0 + kInPT <= nk) {
-      const uint4 v = __ldcs(reinterpret_cast<const uint4 *>(pe));
-      pk[0] = v.x;
-      pk[1] = v.y;
-      pk[2] = v.z;
-      pk[3] = v.w;
-#pragma unroll
-      for (int k = 0; k < kInPT; k += 2) {
-        const uint4 w = __ldcs(reinterpret_cast<const uint4 *>(ke + k));
-        xk[k] = ((u64)w.y << 32) | w.x;
-        xk[k + 1] = ((u64)w.w << 32) | w.z;
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < kInPT; k++) {
-        pk[k] = e0 + k < nk ? __ldcs(pe + k) : ~0u;
-        xk[k] = e0 + k < nk ? __ldcs(ke + k) : 0;
-      }
-    }
-    unsigned bal[kInPT], tot = 0;
-    bool keep[kInPT];
-#pragma unroll
-    for (int k = 0; k < kInPT; k++) {
-      const unsigned p = pk[k];
-      keep[k] = p != ~0u && !((segA[p >> 6] >> (p & 63)) & 1ull);
-      bal[k] = __ballot_sync(0xffffffffu, keep[k]);
-      tot += __popc(bal[k]);
-    }
-    // one reservation per warp and unit in the rotating counter of this unit
-    unsigned wbase = 0;
-    if (lane == 0 && tot) wbase = atomicAdd(&scnt[it % 3], tot);
-    wbase = ns + __shfl_sync(0xffffffffu, wbase, 0);
-#pragma unroll
-    for (int k = 0; k < kInPT; k++) {
-      if (keep[k]) stage[wbase + __popc(bal[k] & lt)] = xk[k];
-      wbase += __popc(bal[k]);
-    }
-    // the counter of unit it+1 was last read after the barrier of unit it-2,
-    // which every thread has passed: reset it for the next unit
-    if (threadIdx.x == 0) scnt[(it + 1) % 3] = 0;
-    __syncthreads();
-    ns += scnt[it % 3];
-    // 2.+3. a full tile of survivors: hash and write it; the survivors past it
-    // (fewer than kIn, beyond the multisplit's part of the stage) move to the
-    // front for the next tile
-    if (ns >= (unsigned)kTile) {
-      flush(kTile);
-      const unsigned left = ns - kTile;
-      for (unsigned i = threadIdx.x; i < left; i += kTT) stage[i] = stage[kTile + i];
-      __syncthreads();
-      ns = left;
-    }
-  }
-  if (ns) flush(ns);
+// A fallback too large for the tail: the values h_{L-1} of F back to keys.
+__global__ void k_unhash(u64 *__restrict__ F, u64 n, u64 s) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
+    F[i] = unmix64(F[i]) ^ s;
 }
 
 // ---------------------------------------------------------------------------
@@ -455,7 +309,7 @@ k_tail(FastMeta *__restrict__ meta, int dlim, FastCfg cfg, u64 mcap) {
     return;
   }
   const u64 n = lvs[t].n;
-  if (threadIdx.x == 0 && meta->n_flat != n) atomicOr(&meta->status, ST_INTERNAL);
+  if (threadIdx.x == 0 && t > 0 && meta->n_out[t - 1] != n) atomicOr(&meta->status, ST_INTERNAL);
   if ((uint32_t)t == cfg.L && n > kTailMaxKeys) {
     // large fallback: sorted on the host side of the build (sort.cu)
     if (threadIdx.x == 0) {
@@ -466,11 +320,14 @@ k_tail(FastMeta *__restrict__ meta, int dlim, FastCfg cfg, u64 mcap) {
     return;
   }
   TailSmem sm = carve_tail(smem, mcap);
-  for (unsigned i = threadIdx.x; i < n; i += kTailThreads) sm.keys[i] = cfg.flat[i];
+  // F holds the values of the level before (at t = 0 the caller's keys)
+  const u64 s_b = t > 0 ? level_seed(cfg.seed, t - 1) : 0;
+  for (unsigned i = threadIdx.x; i < n; i += kTailThreads)
+    sm.keys[i] = t > 0 ? unmix64(cfg.F[i]) ^ s_b : cfg.F[i];
   __syncthreads();
   unsigned used = cta_levels<kTailThreads, (int)kTailMaxKeys>(
       sm, n, t, lvs[t].off, lvs, cfg.gamma, cfg.L, cfg.seed, cfg.A0,
-                             cfg.arena, cfg.m0, cfg.arena_words, cfg.flat, &meta->n_fb,
+                             cfg.arena, cfg.m0, cfg.arena_words, cfg.F, &meta->n_fb,
                              &meta->status);
   if (threadIdx.x == 0) {
     meta->levels_used = used;
@@ -483,26 +340,32 @@ k_tail(FastMeta *__restrict__ meta, int dlim, FastCfg cfg, u64 mcap) {
 // ---------------------------------------------------------------------------
 static bool g_attr_set = false;
 double g_cap_scale = 1.0;
-static size_t g_split_bytes, g_compact_bytes;
+
+using SplitFn = void (*)(const u64 *, u64, FastMeta *, int, FastCfg, unsigned);
+static SplitFn split_fn(unsigned nb_max, bool first) {
+  if (nb_max <= (unsigned)kWT) return first ? k_split<1, true> : k_split<1, false>;
+  return first ? k_split<2, true> : k_split<2, false>;
+}
 
 static int set_attrs() {
   if (g_attr_set) return MPHF_OK;
-
-  g_split_bytes = split_smem_bytes((unsigned)kBmax);
-  // compaction: its largest layout (kBmax destinations) + the bucket's slice of A_d
-  g_compact_bytes = split_smem_bytes((unsigned)kBmax, kTile + kIn) + kPmax / 8;
-  MPHF_CUDA(cudaFuncSetAttribute(k_partition0<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(g_split_bytes + kTile * 8)));
-  MPHF_CUDA(cudaFuncSetAttribute(k_partition0<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(g_split_bytes + kTile * 8)));
-  MPHF_CUDA(cudaFuncSetAttribute(k_compact_buckets, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)g_compact_bytes));
-  MPHF_CUDA(cudaFuncSetAttribute(k_fill_buckets, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  for (int v = 0; v < 4; v++)
+    MPHF_CUDA(cudaFuncSetAttribute(split_fn(v & 1 ? kWMaxNb : 1, (v & 2) != 0),
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWSmem));
+  MPHF_CUDA(cudaFuncSetAttribute(k_fill_compact, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(kPmax / 4)));
   MPHF_CUDA(cudaFuncSetAttribute(k_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  200 * 1024));
   g_attr_set = true;
   return MPHF_OK;
+}
+
+// One split launch of (at most) n values into at most nb_max buckets.
+static void launch_split(const u64 *keys, u64 n, FastMeta *meta, int d, const FastCfg &cfg,
+                         unsigned nb_max, cudaStream_t st) {
+  const unsigned g = grid_for(n, kWT, (unsigned)sm_count());
+  LaunchScope ls("split", st);
+  split_fn(nb_max, d == 0)<<<g, kWT, kWSmem, st>>>(keys, n, meta, d, cfg, nb_max);
 }
 
 // Expected |F_{d+1}| from |F_d| (a key is alone with probability (1 - 1/m)^(n-1)).
@@ -512,11 +375,10 @@ static double expect_next(double n, double gamma) {
 }
 
 struct FastScratch {
-  DevBuf meta, X, Y, XP, YP, cntX, cntY, flat, A0, arena, upre;
+  DevBuf meta, X, cnt, F, A0, arena;
   void release(cudaStream_t s) {
-    dev_free(upre, s);
-    dev_free(meta, s); dev_free(X, s); dev_free(Y, s); dev_free(XP, s); dev_free(YP, s);
-    dev_free(cntX, s); dev_free(cntY, s); dev_free(flat, s); dev_free(A0, s); dev_free(arena, s);
+    dev_free(meta, s); dev_free(X, s); dev_free(cnt, s); dev_free(F, s);
+    dev_free(A0, s); dev_free(arena, s);
   }
 };
 
@@ -524,7 +386,7 @@ struct FastScratch {
 // size the device may pick for |F_1| <= n1_hi = E|F_1| + 10 sqrt(N) + 256
 // (|F_1| has a standard deviation below sqrt(N)).  With B <= Bb buckets of
 // cap = cap_scale (mean + 8 sqrt(mean) + 64) slots, the means summing to at
-// most n + P, B cap <= cap_scale (n + P + 8 sqrt(B (n + P)) + 64 B) + 4 B.
+// most n + P, B cap <= cap_scale (n + P + 8 sqrt(B (n + P)) + 64 B) + 16 B.
 static u64 level1_bound(u64 N, double gamma, u64 Btarget, u64 Pmax, double cap_scale,
                         u64 *n1_hi_out, u64 *Bb_out) {
   const double ev1 = expect_next((double)N, gamma);  // E|F_1|
@@ -536,7 +398,7 @@ static u64 level1_bound(u64 N, double gamma, u64 Btarget, u64 Pmax, double cap_s
   const double tot = (double)(n1_hi + Pmax);
   *n1_hi_out = n1_hi;
   *Bb_out = Bb;
-  return (u64)(cap_scale * (tot + 8.0 * sqrt((double)Bb * tot) + 64.0 * (double)Bb)) + 4 * Bb + 64;
+  return (u64)(cap_scale * (tot + 8.0 * sqrt((double)Bb * tot) + 64.0 * (double)Bb)) + 16 * Bb + 64;
 }
 
 // Largest level size the tail may take for this gamma (keys + 2 bit arrays in 200 KB).
@@ -583,7 +445,6 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
   FastMeta *meta = nullptr;
   int dlim = 0;
   int D = 1;  // levels (from 0) launched before the first look at the device's progress
-  size_t comp_bytes = g_compact_bytes;  // compaction's shared memory for this build
 
 #define FTRY(x)                    \
   do {                             \
@@ -608,16 +469,15 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
     hm.lv[0].n = N;
     hm.lv[0].m = m0;
     hm.lv[0].mode = LM_FLAT;
-    hm.n_flat = N;
-    FTRY(dev_alloc(sc.flat, N * 8, st));
-    cfg.flat = (u64 *)sc.flat.p;
-    cfg.flat_cap = N;
+    FTRY(dev_alloc(sc.F, N * 8, st));
+    cfg.F = (u64 *)sc.F.p;
+    cfg.F_cap = N;
     u64 arena_words = (u64)(L > 1 ? L - 1 : 1) * (level_bits(N, gamma) / 64);
     FTRY(dev_alloc(sc.arena, arena_words * 8, st));
     cfg.arena = (u64 *)sc.arena.p;
     cfg.arena_words = arena_words;
     if (feed) FTRY(feed->ensure(N, st));
-    FCUDA(cudaMemcpyAsync(cfg.flat, keys, N * 8, cudaMemcpyDeviceToDevice, st));
+    FCUDA(cudaMemcpyAsync(cfg.F, keys, N * 8, cudaMemcpyDeviceToDevice, st));
     FCUDA(cudaMemcpyAsync(meta, &hm, sizeof(hm), cudaMemcpyHostToDevice, st));
     {
       LaunchScope ls("tail", st);
@@ -633,105 +493,70 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
       sc.release(st);
       return MPHF_OK;
     }
+    // Levels past the first are sized on the device by the last CTA of the
+    // level before; their buffers come from a bound on |F_1| so that no host
+    // round trip sits between the levels.  |F_1| (keys not alone in their bin
+    // at level 0) has mean N - N (1 - 1/m_0)^(N-1) and a standard deviation
+    // below sqrt(N); the bound adds 10 of those, and level1_bound covers the
+    // buckets of any level that small.  A level that does not fit anyway
+    // (duplicate-heavy input) is caught on the device and the build is redone
+    // by the unbucketed path.
+    u64 n1_hi = 0, Bb = 0;
+    const u64 cap1 = level1_bound(N, gamma, cfg.Btarget, cfg.Pmax, cfg.cap_scale, &n1_hi, &Bb);
+    const u64 m1_hi = level_bits(n1_hi, gamma);
     cfg.capX = hm.lv[0].B * hm.lv[0].cap;
+    if (cfg.capX < cap1) cfg.capX = cap1;
     FTRY(dev_alloc(sc.X, cfg.capX * 8, st));
-    FTRY(dev_alloc(sc.XP, cfg.capX * 4, st));
-    cfg.XP = (unsigned *)sc.XP.p;
-    FTRY(dev_alloc(sc.cntX, kBmax * 8, st));
-    FTRY(dev_alloc(sc.cntY, kBmax * 8, st));
-    FTRY(dev_alloc(sc.upre, (kBmax + 1) * 4, st));
-    cfg.upre = (unsigned *)sc.upre.p;
+    FTRY(dev_alloc(sc.cnt, kBmax * 8, st));
     cfg.X = (u64 *)sc.X.p;
-    cfg.cntX = (u64 *)sc.cntX.p;
-    cfg.cntY = (u64 *)sc.cntY.p;
+    cfg.cnt = (u64 *)sc.cnt.p;
+    cfg.F_cap = n1_hi < T ? T : n1_hi;
+    FTRY(dev_alloc(sc.F, cfg.F_cap * 8, st));
+    cfg.F = (u64 *)sc.F.p;
+    cfg.arena_words = (u64)(L > 1 ? L - 1 : 1) * (m1_hi / 64);
+    FTRY(dev_alloc(sc.arena, cfg.arena_words * 8, st));
+    cfg.arena = (u64 *)sc.arena.p;
+    // level 1 has the most keys of the levels >= 1, and a smaller level never
+    // takes more than Btarget buckets (its width shrinks first), so Bb bounds
+    // them all; the split checks it and falls back if ever exceeded
+    const unsigned nb1 = (unsigned)(Bb < kBmax ? Bb : kBmax);
     {
-      // Level 1 is sized on the device by the last CTA of level 0's fill; its
-      // buffers come from a bound on |F_1| so that no host round trip sits
-      // between the levels.  |F_1| (keys not alone in their bin at level 0)
-      // has mean N - N (1 - 1/m_0)^(N-1) and a standard deviation below
-      // sqrt(N); the bound adds 10 of those.  With n1 <= n1_hi, any level
-      // size the device picks (B buckets of cap slots, B <= Bb) fits
-      //   capY = n1_hi + Pmax + 8 sqrt(Bb (n1_hi + Pmax)) + 64 Bb (+ rounding),
-      // since the bucket means sum to at most n + P and sqrt is concave.  A
-      // level that does not fit anyway (duplicate-heavy input) is caught by
-      // finish_level and the build is redone by the unbucketed path.
-      const double ev1 = expect_next((double)N, gamma);  // E|F_1|
-      u64 n1_hi = 0, Bb = 0;
-      cfg.capY = level1_bound(N, gamma, cfg.Btarget, cfg.Pmax, cfg.cap_scale, &n1_hi, &Bb);
-      const u64 m1_hi = level_bits(n1_hi, gamma);
-      FTRY(dev_alloc(sc.Y, cfg.capY * 8, st));
-      FTRY(dev_alloc(sc.YP, cfg.capY * 4, st));
-      cfg.Y = (u64 *)sc.Y.p;
-      cfg.YP = (unsigned *)sc.YP.p;
-      cfg.flat_cap = n1_hi < (1ull << 22) ? n1_hi : (1ull << 22);
-      if (cfg.flat_cap < T) cfg.flat_cap = T;
-      FTRY(dev_alloc(sc.flat, cfg.flat_cap * 8, st));
-      cfg.flat = (u64 *)sc.flat.p;
-      cfg.arena_words = (u64)(L > 1 ? L - 1 : 1) * (m1_hi / 64);
-      FTRY(dev_alloc(sc.arena, cfg.arena_words * 8, st));
-      cfg.arena = (u64 *)sc.arena.p;
-      // destination buckets of any compaction: level 1 has the most keys of
-      // the levels >= 1, and a smaller level never takes more than Btarget
-      // buckets (its width shrinks first), so Bb bounds them all; the
-      // compaction checks it and falls back if ever exceeded
-      cfg.nbcap = Bb < kBmax ? Bb : kBmax;
-      comp_bytes = split_smem_bytes((unsigned)cfg.nbcap, kTile + kIn) + kPmax / 8;
-      // predicted number of bucketed levels after level 0
-      double e = ev1;
+      // predicted number of bucketed levels
+      double e = expect_next((double)N, gamma);
       D = 1;
       while (e > (double)T && D < (int)L) {
         e = expect_next(e, gamma);
         D++;
       }
     }
-    FCUDA(cudaMemsetAsync(sc.cntX.p, 0, kBmax * 8, st));
+    FCUDA(cudaMemsetAsync(sc.cnt.p, 0, kBmax * 8, st));
     FCUDA(cudaMemcpyAsync(meta, &hm, sizeof(hm), cudaMemcpyHostToDevice, st));
-    // Level-0 partition.  Keys still arriving from the host are partitioned
-    // one chunk per launch as each chunk lands (the buckets' counters only
-    // grow, so the launches compose); chunk starts are multiples of kTile.
+    // Level-0 split.  Keys still arriving from the host are split one chunk
+    // per launch as each chunk lands (the buckets' counters only grow, so the
+    // launches compose).
     const u64 pstep = feed && feed->chunk ? feed->chunk : N;
     for (u64 c0 = 0; c0 < N; c0 += pstep) {
       const u64 cn = N - c0 < pstep ? N - c0 : pstep;
       if (feed) FTRY(feed->ensure(c0 + cn, st));
-      const u64 *kc = keys + c0;
-      const unsigned gridP = grid_for(cn, kTile, (unsigned)sm_count() * 2);
-      LaunchScope ls("partition", st);
-      if (((uintptr_t)kc & 15) == 0)
-        k_partition0<true><<<gridP, kTT, g_split_bytes + kTile * 8, st>>>(kc, cn, meta, cfg);
-      else
-        k_partition0<false><<<gridP, kTT, g_split_bytes + kTile * 8, st>>>(kc, cn, meta, cfg);
+      launch_split(keys + c0, cn, meta, 0, cfg, (unsigned)hm.lv[0].B, st);
     }
-    {
-      LaunchScope ls("fill_buckets", st);
-      k_fill_buckets<<<(unsigned)(hm.lv[0].B < (u64)sm_count() * 2 ? hm.lv[0].B
-                                                                    : (u64)sm_count() * 2),
-                       kTT,
-                       (size_t)(hm.lv[0].P / 4), st>>>(meta, 0, cfg);
-    }
-    FCUDA(cudaGetLastError());
-    {
-      for (int round = 0; round < 64; round++) {
-        for (; dlim < D && dlim < (int)L; dlim++) {
-          {
-            LaunchScope ls("compact_buckets", st);
-            k_compact_buckets<<<(unsigned)sm_count() * 2, kTT, comp_bytes, st>>>(meta, dlim, cfg);
-          }
-          if (dlim + 1 < (int)L) {
-            LaunchScope ls("fill_buckets", st);
-            k_fill_buckets<<<(unsigned)sm_count() * 2, kTT, (size_t)(cfg.Pmax / 4), st>>>(
-                meta, dlim + 1, cfg);
-          }
-        }
-        {
-          LaunchScope ls("tail", st);
-          k_tail<<<1, kTailThreads, tail_smem_bytes(mcap), st>>>(meta, dlim, cfg, mcap);
-        }
-        FCUDA(cudaGetLastError());
-        FCUDA(cudaMemcpyAsync(&hm, meta, sizeof(hm), cudaMemcpyDeviceToHost, st));
-        FCUDA(cudaStreamSynchronize(st));
-        if (hm.status || hm.tail_done || dlim >= (int)L) break;
-        D = dlim + 2;
+    const unsigned ctas = (unsigned)sm_count() * 2;
+    for (int round = 0; round < 64; round++) {
+      for (; dlim < D && dlim < (int)L; dlim++) {
+        if (dlim > 0) launch_split(nullptr, n1_hi, meta, dlim, cfg, nb1, st);
+        LaunchScope ls("fill_compact", st);
+        k_fill_compact<<<dlim == 0 && hm.lv[0].B < ctas ? (unsigned)hm.lv[0].B : ctas, kTT,
+                         (size_t)((dlim == 0 ? hm.lv[0].P : cfg.Pmax) / 4), st>>>(meta, dlim, cfg);
       }
+      {
+        LaunchScope ls("tail", st);
+        k_tail<<<1, kTailThreads, tail_smem_bytes(mcap), st>>>(meta, dlim, cfg, mcap);
+      }
+      FCUDA(cudaGetLastError());
+      FCUDA(cudaMemcpyAsync(&hm, meta, sizeof(hm), cudaMemcpyDeviceToHost, st));
+      FCUDA(cudaStreamSynchronize(st));
+      if (hm.status || hm.tail_done || dlim >= (int)L) break;
+      D = dlim + 2;
     }
   }
   if (N <= T) {
@@ -780,9 +605,16 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
                       &meta->rank_total, st));
     unsigned *dflag = &meta->dup;
     if (n_fb) {
-      if (hm.tail_done == 2) FTRY(sort_fallback(cfg.flat, n_fb, dflag, st));
+      if (hm.tail_done == 2) {
+        {
+          LaunchScope ls("unhash", st);
+          k_unhash<<<grid_for(n_fb, 256 * 4, (unsigned)sm_count() * 8), 256, 0, st>>>(
+              cfg.F, n_fb, level_seed(seed, L - 1));
+        }
+        FTRY(sort_fallback(cfg.F, n_fb, dflag, st));
+      }
       FTRY(dev_alloc(h->fb, n_fb * 8, st));
-      FCUDA(cudaMemcpyAsync(h->fb.p, cfg.flat, n_fb * 8, cudaMemcpyDeviceToDevice, st));
+      FCUDA(cudaMemcpyAsync(h->fb.p, cfg.F, n_fb * 8, cudaMemcpyDeviceToDevice, st));
     }
     FCUDA(cudaMemcpyAsync(&hm, meta, sizeof(hm), cudaMemcpyDeviceToHost, st));
     FCUDA(cudaStreamSynchronize(st));

@@ -9,8 +9,8 @@ namespace bbh {
 // Where the keys of level d live.
 enum LevelMode : unsigned {
   LM_NONE = 0,
-  LM_BUCKETED = 1,  // in position-range buckets of arena (d & 1)
-  LM_FLAT = 2,      // contiguous in the flat buffer (input of the tail, or the fallback if d == L)
+  LM_BUCKETED = 1,  // in position-range buckets
+  LM_FLAT = 2,      // contiguous in F (input of the tail, or the fallback if d == L)
   LM_DONE = 3       // no keys left: the function ends at level d - 1
 };
 
@@ -33,7 +33,7 @@ struct FLevel {
 struct FastMeta {
   FLevel lv[MPHF_MAX_LEVELS + 1];
   u64 seen[MPHF_MAX_LEVELS + 1];  // keys found in the buckets of level d (consistency check)
-  u64 n_flat;            // keys appended to the flat buffer
+  u64 n_out[MPHF_MAX_LEVELS + 1]; // keys written to F_{d+1} by level d's compaction
   u64 n_fb;              // fallback keys
   u64 rank_total;        // ones of A, from the rank table
   unsigned status;
@@ -47,13 +47,12 @@ struct FastCfg {
   double gamma;
   uint32_t L;
   u64 seed;
-  u64 *X, *Y;           // bucket arenas: levels with even / odd d
-  unsigned *XP, *YP;    // in-bucket position of each key of X / Y
-  u64 capX, capY;       // their capacities in keys
-  u64 *cntX, *cntY;     // per-bucket key counts
-  u64 Bmax;             // capacity of the count arrays
-  u64 *flat;            // flat buffer (tail input / fallback)
-  u64 flat_cap;
+  u64 *X;               // bucket arena: the current level's values h_d, by bucket
+  u64 capX;             // its capacity in values
+  u64 *cnt;             // per-bucket counts
+  u64 Bmax;             // capacity of the count array
+  u64 *F;               // F_{d+1} as values h_d (tail input / fallback at the end)
+  u64 F_cap;
   u64 *A0;              // A_0 (m_0 bits)
   u64 *arena;           // A_1, A_2, ... back to back
   u64 m0;
@@ -61,8 +60,6 @@ struct FastCfg {
   u64 T;                // levels with at most T keys run in the single-CTA tail
   u64 Pmax, Pmin, Btarget;
   double cap_scale;     // bucket capacity multiplier (1 in production; < 1 only in tests)
-  unsigned *upre;       // [Bmax + 1] compaction units (kIn-entry slices) before each bucket
-  u64 nbcap;            // compaction: capacity of its per-destination-bucket arrays
 };
 
 __host__ __device__ inline u64 ceil_div(u64 a, u64 b) { return (a + b - 1) / b; }
@@ -97,7 +94,7 @@ __host__ __device__ inline void size_bucketed(FLevel &lv, u64 n, double gamma, u
   lv.B = ceil_div(lv.m, P);
   double mean = (double)n * (double)P / (double)lv.m;
   u64 cap = (u64)(cap_scale * (mean + 8.0 * sqrt(mean) + 64.0));
-  lv.cap = (cap + 3) & ~3ull;  // multiple of 4: every bucket starts 16-byte aligned
+  lv.cap = (cap + 15) & ~15ull;  // every bucket starts on a 128-byte line
 }
 
 // ---------------------------------------------------------------------------
