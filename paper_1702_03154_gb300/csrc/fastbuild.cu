@@ -28,8 +28,9 @@
 // ms for level 0, 0.32 + 1.02 ms for fills and compactions, 2.34 ms in all.
 #include <cuda_runtime.h>
 #include <math.h>
-#include <stdlib.h>
 #include <string.h>
+
+#include <algorithm>
 
 #include "fastbuild.cuh"
 #include "sector.cuh"
@@ -37,6 +38,12 @@
 
 namespace bbh {
 
+
+// Position of hash value y in A_d, modulo 2^32 (NARROW: m < 2^32).
+template <bool NARROW>
+__device__ __forceinline__ unsigned position(u64 y, u64 m) {
+  return NARROW ? reduce_range32(y, (unsigned)m) : (unsigned)__umul64hi(y, m);
+}
 
 // Split of level d: the caller's keys (d = 0) or the survivors of level d - 1
 // (F, as values h_{d-1}) to the position buckets of A_d, as values h_d.
@@ -53,12 +60,12 @@ k_split(const u64 *__restrict__ keys, u64 n, FastMeta *__restrict__ meta, int d,
     if (threadIdx.x == 0) atomicOr(&meta->status, ST_OVERFLOW);
     return;
   }
-  const WcShape sh = wc_shape((unsigned)lv.B);
+  const WcShape sh = wc_shape((unsigned)lv.B, kWT, wc_smem(1));
   const u64 s_d = level_seed(cfg.seed, d);
   const u64 s_x = FIRST ? s_d : s_d ^ level_seed(cfg.seed, d - 1);
   const unsigned m = (unsigned)lv.m, shift = ilog2_u64(lv.P);
-  wc_split<OWN>(
-      FIRST ? keys : cfg.F, FIRST ? n : lv.n, sh, smem,
+  wc_split<kWT, OWN>(
+      FIRST ? keys : cfg.F, FIRST ? n : lv.n, blockIdx.x, gridDim.x, sh, smem,
       [=](u64 v) { return mix64((FIRST ? v : unmix64(v)) ^ s_x); },
       [=](u64 y) { return reduce_range32(y, m) >> shift; }, UniformDest{cfg.cnt, lv.cap}, cfg.X,
       &meta->status);
@@ -99,39 +106,44 @@ __device__ void finish_level(FastMeta *meta, int d, const FastCfg &cfg) {
 }
 
 // ---------------------------------------------------------------------------
-// ArrayFill (Algorithm 2) and compaction (Algorithm 1) of level d, one bucket
-// per CTA iteration with its hit and collision bits in shared memory.  Pass 1
-// streams the bucket's values and sets the bits; A_d's words of the bucket
-// leave and their ones are counted, which also fixes the number of survivors
-// (values in the bucket less ones), so one global atomic reserves the whole
-// bucket's run of F_{d+1}.  Pass 2 streams the values again and writes those
-// whose bit is 0, each warp taking its part of the run with a shared-memory
-// atomic.  The last CTA sizes level d+1.
+// ArrayFill (Algorithm 2) and compaction (Algorithm 1) of buckets of one
+// level, a bucket per CTA iteration with its hit and collision bits in shared
+// memory.  Pass 1 streams the bucket's values and sets the bits; A_d's words
+// of the bucket leave and their ones are counted, which also fixes the number
+// of survivors (values in the bucket less ones), so one global atomic reserves
+// the whole bucket's run of F_{d+1}.  Pass 2 streams the values again, last
+// first, and writes those whose bit is 0, each warp taking its part of the run
+// with a shared-memory atomic.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kTT, 2)
-k_fill_compact(FastMeta *__restrict__ meta, int d, FastCfg cfg) {
-  extern __shared__ __align__(16) unsigned char smem[];
+struct FillArgs {
+  const u64 *X;    // values, bucket b at [b cap, b cap + cnt[b])
+  const u64 *cnt;
+  u64 cap, B;      // slots of a bucket, buckets
+  u64 m, P, p0;    // |A_d|; positions of a bucket; first position of bucket 0
+  u64 *A;          // A_d
+  u64 *F, F_cap, *n_out;
+  unsigned *status;
+};
+
+// Adds the ones of the CTA's buckets and the values found in them to wtot and
+// got (thread 0).
+template <bool NARROW>
+__device__ __forceinline__ void fill_compact(const FillArgs &a, unsigned char *smem, u64 &wtot,
+                                             u64 &got) {
   __shared__ u64 red[kTT / 32];
   __shared__ u64 s_base;
   __shared__ unsigned s_count, s_room;
-  __shared__ bool last;
-  if (__syncthreads_or(meta->lv[d].mode != LM_BUCKETED || *(volatile unsigned *)&meta->status))
-    return;
-  const FLevel lv = meta->lv[d];
-  u64 *Alev = (d == 0) ? cfg.A0 : cfg.arena + ((lv.off - cfg.m0) >> 6);
-  const unsigned Pw = (unsigned)(lv.P >> 5);  // 32-bit words per bit array
+  const unsigned Pw = (unsigned)(a.P >> 5);  // 32-bit words per bit array
   unsigned *hit = reinterpret_cast<unsigned *>(smem);
   unsigned *col = hit + Pw;
-  const unsigned m = (unsigned)lv.m;
   const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
-  u64 wtot = 0, got = 0;  // thread 0: ones and values of this CTA's buckets
-  for (u64 b = blockIdx.x; b < lv.B; b += gridDim.x) {
+  for (u64 b = blockIdx.x; b < a.B; b += gridDim.x) {
     for (unsigned i = threadIdx.x; i < Pw / 2; i += kTT)
       reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0, 0, 0, 0);
-    const unsigned nk = (unsigned)min(cfg.cnt[b], lv.cap);
-    const u64 *yb = cfg.X + b * lv.cap;
+    const unsigned nk = (unsigned)min(a.cnt[b], a.cap);
+    const u64 *yb = a.X + b * a.cap;
     const uint4 *y4 = reinterpret_cast<const uint4 *>(yb);  // cap % 16 == 0
-    const unsigned p0 = (unsigned)(b * lv.P);
+    const unsigned p0 = (unsigned)(a.p0 + b * a.P);  // positions modulo 2^32
     const unsigned nv = nk >> 1;  // pairs of values
     auto val0 = [](const uint4 &v) { return ((u64)v.y << 32) | v.x; };
     auto val1 = [](const uint4 &v) { return ((u64)v.w << 32) | v.z; };
@@ -147,7 +159,7 @@ k_fill_compact(FastMeta *__restrict__ meta, int d, FastCfg cfg) {
                      "r"(min(kStep, nv - s * kStep) * 16));
     };
     auto set = [&](u64 y) {
-      const unsigned q = reduce_range32(y, m) - p0;
+      const unsigned q = position<NARROW>(y, a.m) - p0;
       const unsigned bit = 1u << (q & 31);
       const unsigned old = atomicOr(hit + (q >> 5), bit);
       if (old & bit) atomicOr(col + (q >> 5), bit);
@@ -172,16 +184,16 @@ k_fill_compact(FastMeta *__restrict__ meta, int d, FastCfg cfg) {
     }
     if ((nk & 1) && threadIdx.x == 0) set(yb[nk - 1]);
     __syncthreads();
-    // A_d words of this bucket: positions [b P, min((b+1) P, m)); hit keeps A
-    const u64 w0 = (b * lv.P) >> 6;
-    const unsigned nw = (unsigned)((min((b + 1) * lv.P, lv.m) >> 6) - w0);
+    // A_d words of this bucket's positions; hit keeps A
+    const u64 w0 = (a.p0 + b * a.P) >> 6;
+    const unsigned nw = (unsigned)((min(a.p0 + (b + 1) * a.P, a.m) >> 6) - w0);
     unsigned wsum = 0;
     for (unsigned w = threadIdx.x; w < nw; w += kTT) {
       const uint2 h2 = reinterpret_cast<uint2 *>(hit)[w], c2 = reinterpret_cast<uint2 *>(col)[w];
-      const uint2 a = make_uint2(h2.x & ~c2.x, h2.y & ~c2.y);
-      reinterpret_cast<uint2 *>(hit)[w] = a;
-      Alev[w0 + w] = ((u64)a.y << 32) | a.x;
-      wsum += __popc(a.x) + __popc(a.y);
+      const uint2 k2 = make_uint2(h2.x & ~c2.x, h2.y & ~c2.y);
+      reinterpret_cast<uint2 *>(hit)[w] = k2;
+      a.A[w0 + w] = ((u64)k2.y << 32) | k2.x;
+      wsum += __popc(k2.x) + __popc(k2.y);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) wsum += __shfl_down_sync(0xffffffffu, wsum, o);
@@ -191,22 +203,22 @@ k_fill_compact(FastMeta *__restrict__ meta, int d, FastCfg cfg) {
       u64 w = 0;
       for (int i = 0; i < kTT / 32; i++) w += red[i];
       wtot += w;
-      got += cfg.cnt[b];
+      got += a.cnt[b];
       const u64 ns = w > nk ? 0 : nk - w;
-      const u64 at = ns ? atomicAdd(&meta->n_out[d], ns) : 0;
-      const bool fits = w <= nk && at + ns <= cfg.F_cap;
-      if (!fits) atomicOr(&meta->status, ST_OVERFLOW);
+      const u64 at = ns ? atomicAdd(a.n_out, ns) : 0;
+      const bool fits = w <= nk && at + ns <= a.F_cap;
+      if (!fits) atomicOr(a.status, ST_OVERFLOW);
       s_base = at;
       s_room = fits ? (unsigned)ns : 0u;
       s_count = 0;
     }
     __syncthreads();
-    u64 *out = cfg.F + s_base;
+    u64 *out = a.F + s_base;
     const unsigned room = s_room;
     // pass 2, last step first (it is the likeliest to be still in L2): a warp
     // step takes U groups of 32 pairs
     auto kept = [&](u64 y) {
-      const unsigned q = reduce_range32(y, m) - p0;
+      const unsigned q = position<NARROW>(y, a.m) - p0;
       return !((hit[q >> 5] >> (q & 31)) & 1u);
     };
     for (unsigned st = nsteps; st-- > 0;) {
@@ -246,6 +258,21 @@ k_fill_compact(FastMeta *__restrict__ meta, int d, FastCfg cfg) {
     }
     __syncthreads();
   }
+}
+
+// Level d of the device-driven loop; the last CTA sizes level d+1.
+__global__ void __launch_bounds__(kTT, 2)
+k_fill_compact(FastMeta *__restrict__ meta, int d, FastCfg cfg) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ bool last;
+  if (__syncthreads_or(meta->lv[d].mode != LM_BUCKETED || *(volatile unsigned *)&meta->status))
+    return;
+  const FLevel lv = meta->lv[d];
+  u64 *Alev = (d == 0) ? cfg.A0 : cfg.arena + ((lv.off - cfg.m0) >> 6);
+  u64 wtot = 0, got = 0;
+  fill_compact<true>(FillArgs{cfg.X, cfg.cnt, lv.cap, lv.B, lv.m, lv.P, 0, Alev, cfg.F, cfg.F_cap,
+                              &meta->n_out[d], &meta->status},
+                     smem, wtot, got);
   if (threadIdx.x == 0) {
     if (wtot) atomicAdd(&meta->lv[d].weight, wtot);
     if (got) atomicAdd(&meta->seen[d], got);
@@ -266,6 +293,78 @@ k_fill_compact(FastMeta *__restrict__ meta, int d, FastCfg cfg) {
     const FLevel nx = meta->lv[d + 1];
     if (nx.mode == LM_BUCKETED)
       for (u64 i = threadIdx.x; i < nx.B; i += kTT) cfg.cnt[i] = 0;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Levels with more buckets than one split takes well are grouped in two
+// steps: all values to coarse slabs of 2^cs positions (k_gsplit),
+// then, a batch of slabs at a time, each slab's values to its fine buckets of
+// 2^kGroupShift positions (k_fsplit: a group of CTAs per slab) and the batch's
+// buckets filled and compacted (k_gfill).  Measured at 3e9 keys (gamma = 2):
+// coarse 20.4 ms, fine 19.5, fill and compaction 15.7 for the three grouped
+// levels (4.6e9 values, 16 bytes a split), build 60 ms; counting-sort
+// multisplits and a fill from stored positions took 54.5 + 23.1 ms, build 81.
+// ---------------------------------------------------------------------------
+static constexpr unsigned kGroupShift = 17;
+static constexpr unsigned kBatchFine = 2048;  // fine buckets per batch
+
+// Coarse slabs of a level of m positions: 2^shift positions each, so that the
+// two splits have about as many destinations (a third or three times as many
+// slabs: within 3% at 3e9 keys).
+static unsigned coarse_shift(u64 m) {
+  unsigned sh = kGroupShift;
+  while (ceil_div(m, 1ull << sh) > 1ull << (sh - kGroupShift) && sh < kGroupShift + 9) sh++;
+  return sh;
+}
+// Group a level of more buckets than one split takes.  Both sides measured at
+// 2.6e8 keys (gamma 2, 1984 buckets): one split 5.3 ms a build, two steps 6.1.
+static constexpr u64 kGroupMinB = kBmax;
+
+template <int NT, bool FIRST, bool NARROW>
+__global__ void __launch_bounds__(NT, kWT / NT)
+k_gsplit(const u64 *__restrict__ in, u64 n, u64 m, unsigned cs, u64 s_x, unsigned nb,
+         u64 *__restrict__ cnt, u64 cap, u64 *__restrict__ out, unsigned *__restrict__ status) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  wc_split<NT, 1>(
+      in, n, blockIdx.x, gridDim.x, wc_shape(nb, NT, wc_smem(kWT / NT)), smem,
+      [=](u64 v) { return mix64((FIRST ? v : unmix64(v)) ^ s_x); },
+      [=](u64 y) {
+        return NARROW ? reduce_range32(y, (unsigned)m) >> cs : (unsigned)(__umul64hi(y, m) >> cs);
+      },
+      UniformDest{cnt, cap}, out, status);
+}
+
+// Slabs [s0, s0 + ns) of R (cap_c slots each) into fine buckets of cap_f
+// slots; gridDim.x = ns * (CTAs a slab).
+template <int NT, bool NARROW>
+__global__ void __launch_bounds__(NT, kWT / NT)
+k_fsplit(const u64 *__restrict__ R, const u64 *__restrict__ cnt_c, u64 cap_c, unsigned s0,
+         unsigned ns, unsigned nf, u64 m, u64 *__restrict__ cnt_f, u64 cap_f, u64 *__restrict__ T,
+         unsigned *__restrict__ status) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const unsigned per = gridDim.x / ns, j = blockIdx.x / per;
+  const u64 n = min(cnt_c[s0 + j], cap_c);
+  const unsigned f0 = (s0 + j) * nf;  // the slab's first fine bucket
+  wc_split<NT, 1>(
+      R + (s0 + j) * cap_c, n, blockIdx.x - j * per, per, wc_shape(nf, NT, wc_smem(kWT / NT)), smem,
+      [](u64 v) { return v; },
+      [=](u64 y) {
+        return (NARROW ? reduce_range32(y, (unsigned)m) >> kGroupShift
+                       : (unsigned)(__umul64hi(y, m) >> kGroupShift)) - f0;
+      },
+      UniformDest{cnt_f + j * nf, cap_f}, T + (u64)j * nf * cap_f, status);
+}
+
+template <bool NARROW>
+__global__ void __launch_bounds__(kTT, 2)
+k_gfill(FillArgs a, u64 *__restrict__ weight, u64 *__restrict__ seen) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  u64 wtot = 0, got = 0;
+  fill_compact<NARROW>(a, smem, wtot, got);
+  if (threadIdx.x == 0) {
+    if (wtot) atomicAdd(weight, wtot);
+    if (got) atomicAdd(seen, got);
   }
 }
 
@@ -347,13 +446,43 @@ static SplitFn split_fn(unsigned nb_max, bool first) {
   return first ? k_split<2, true> : k_split<2, false>;
 }
 
+using GsplitFn = void (*)(const u64 *, u64, u64, unsigned, u64, unsigned, u64 *, u64, u64 *,
+                          unsigned *);
+template <int NT>
+static GsplitFn gsplit_nt(bool first, bool narrow) {
+  if (first) return narrow ? k_gsplit<NT, true, true> : k_gsplit<NT, true, false>;
+  return narrow ? k_gsplit<NT, false, true> : k_gsplit<NT, false, false>;
+}
+static GsplitFn gsplit_fn(int nt, bool first, bool narrow) {
+  return nt == kWT ? gsplit_nt<kWT>(first, narrow) : gsplit_nt<kWT / 2>(first, narrow);
+}
+using FsplitFn = void (*)(const u64 *, const u64 *, u64, unsigned, unsigned, unsigned, u64, u64 *,
+                          u64, u64 *, unsigned *);
+static FsplitFn fsplit_fn(int nt, bool narrow) {
+  if (nt == kWT) return narrow ? k_fsplit<kWT, true> : k_fsplit<kWT, false>;
+  return narrow ? k_fsplit<kWT / 2, true> : k_fsplit<kWT / 2, false>;
+}
+
 static int set_attrs() {
   if (g_attr_set) return MPHF_OK;
   for (int v = 0; v < 4; v++)
     MPHF_CUDA(cudaFuncSetAttribute(split_fn(v & 1 ? kWMaxNb : 1, (v & 2) != 0),
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWSmem));
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wc_smem(1)));
   MPHF_CUDA(cudaFuncSetAttribute(k_fill_compact, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(kPmax / 4)));
+  for (int v = 0; v < 8; v++) {
+    const int nt = v & 4 ? kWT : kWT / 2;
+    MPHF_CUDA(cudaFuncSetAttribute(gsplit_fn(nt, v & 1, v & 2),
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)wc_smem(kWT / nt)));
+    MPHF_CUDA(cudaFuncSetAttribute(fsplit_fn(nt, v & 1),
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)wc_smem(kWT / nt)));
+  }
+  MPHF_CUDA(cudaFuncSetAttribute(k_gfill<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 1 << (kGroupShift - 2)));
+  MPHF_CUDA(cudaFuncSetAttribute(k_gfill<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 1 << (kGroupShift - 2)));
   MPHF_CUDA(cudaFuncSetAttribute(k_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  200 * 1024));
   g_attr_set = true;
@@ -365,7 +494,7 @@ static void launch_split(const u64 *keys, u64 n, FastMeta *meta, int d, const Fa
                          unsigned nb_max, cudaStream_t st) {
   const unsigned g = grid_for(n, kWT, (unsigned)sm_count());
   LaunchScope ls("split", st);
-  split_fn(nb_max, d == 0)<<<g, kWT, kWSmem, st>>>(keys, n, meta, d, cfg, nb_max);
+  split_fn(nb_max, d == 0)<<<g, kWT, wc_smem(1), st>>>(keys, n, meta, d, cfg, nb_max);
 }
 
 // Expected |F_{d+1}| from |F_d| (a key is alone with probability (1 - 1/m)^(n-1)).
@@ -375,10 +504,10 @@ static double expect_next(double n, double gamma) {
 }
 
 struct FastScratch {
-  DevBuf meta, X, cnt, F, A0, arena;
+  DevBuf meta, X, cnt, F, A0, arena, T;
   void release(cudaStream_t s) {
     dev_free(meta, s); dev_free(X, s); dev_free(cnt, s); dev_free(F, s);
-    dev_free(A0, s); dev_free(arena, s);
+    dev_free(A0, s); dev_free(arena, s); dev_free(T, s);
   }
 };
 
@@ -399,6 +528,121 @@ static u64 level1_bound(u64 N, double gamma, u64 Btarget, u64 Pmax, double cap_s
   *n1_hi_out = n1_hi;
   *Bb_out = Bb;
   return (u64)(cap_scale * (tot + 8.0 * sqrt((double)Bb * tot) + 64.0 * (double)Bb)) + 16 * Bb + 64;
+}
+
+// Slots of a bucket that expects `mean` values.
+static u64 group_cap(double mean, double cap_scale) {
+  const u64 cap = (u64)(cap_scale * (mean + 8.0 * sqrt(mean) + 64.0));
+  return (cap + 15) & ~15ull;
+}
+
+// Levels [0, ...) of a build whose level 0 has more than kGroupMinB buckets:
+// runs every level that large, one host round trip per level, and leaves hm
+// with the records of those levels and of the first level after them, whose
+// values are in cfg.F.  *first receives that level's number.
+static int grouped_levels(const u64 *keys, u64 N, const FastCfg &cfg, FastMeta *meta,
+                          FastMeta *hm, FastScratch &sc, int *first, cudaStream_t st) {
+  u64 n = N, off = 0;
+  int d = 0;
+  for (;; d++) {
+    const u64 m = level_bits(n, cfg.gamma);
+    FLevel &lv = hm->lv[d];
+    if (d > 0 && ceil_div(m, cfg.Pmax) <= kGroupMinB) break;
+    lv.n = n;
+    lv.m = m;
+    lv.off = off;
+    lv.mode = LM_BUCKETED;
+    const unsigned cs = coarse_shift(m), nf = 1u << (cs - kGroupShift), batch = kBatchFine / nf;
+    const unsigned nc = (unsigned)ceil_div(m, 1ull << cs);
+    const u64 cap_c = group_cap((double)n * (double)(1ull << cs) / (double)m, cfg.cap_scale);
+    const u64 cap_f =
+        group_cap((double)n * (double)(1ull << kGroupShift) / (double)m, cfg.cap_scale);
+    u64 *cnt_c = (u64 *)sc.cnt.p, *cnt_f = cnt_c + kWMaxNb;
+    if (nc > (unsigned)kWT || nc * cap_c > cfg.capX ||
+        (u64)kBatchFine * cap_f * 8 > sc.T.bytes)
+      return MPHF_EINTERNAL;  // cannot happen: sized for level 0, and levels shrink
+    MPHF_CUDA(cudaMemsetAsync(cnt_c, 0, kWMaxNb * 8, st));
+    const bool narrow = (m >> 32) == 0;
+    const u64 s_d = level_seed(cfg.seed, d);
+    {
+      LaunchScope ls("split_coarse", st);
+      const int nt = wc_threads(nc);
+      gsplit_fn(nt, d == 0, narrow)<<<(unsigned)(sm_count() * (kWT / nt)), nt, wc_smem(kWT / nt),
+                                      st>>>(
+          d == 0 ? keys : cfg.F, n, m, cs, d == 0 ? s_d : s_d ^ level_seed(cfg.seed, d - 1), nc,
+          cnt_c, cap_c, cfg.X, &meta->status);
+    }
+    u64 *Alev = d == 0 ? cfg.A0 : cfg.arena + ((off - cfg.m0) >> 6);
+    for (unsigned s0 = 0; s0 < nc; s0 += batch) {
+      const unsigned ns = nc - s0 < batch ? nc - s0 : batch;
+      MPHF_CUDA(cudaMemsetAsync(cnt_f, 0, (size_t)ns * nf * 8, st));
+      const int nt = wc_threads(nf);
+      const unsigned per = (unsigned)(sm_count() * (kWT / nt)) / ns;
+      {
+        LaunchScope ls("split_fine", st);
+        fsplit_fn(nt, narrow)<<<ns * per, nt, wc_smem(kWT / nt), st>>>(
+            cfg.X, cnt_c, cap_c, s0, ns, nf, m, cnt_f, cap_f, (u64 *)sc.T.p, &meta->status);
+      }
+      FillArgs a;
+      a.X = (const u64 *)sc.T.p;
+      a.cnt = cnt_f;
+      a.cap = cap_f;
+      a.m = m;
+      a.P = 1ull << kGroupShift;
+      a.p0 = (u64)s0 << cs;
+      a.B = ceil_div(std::min((u64)ns << cs, m - a.p0), a.P);
+      a.A = Alev;
+      a.F = cfg.F;
+      a.F_cap = cfg.F_cap;
+      a.n_out = &meta->n_out[d];
+      a.status = &meta->status;
+      {
+        LaunchScope ls("fill_grouped", st);
+        (narrow ? k_gfill<true> : k_gfill<false>)<<<grid_for(a.B, 1, (unsigned)sm_count() * 2), kTT,
+                                                    (size_t)a.P / 4, st>>>(
+            a, &meta->lv[d].weight, &meta->seen[d]);
+      }
+    }
+    MPHF_CUDA(cudaGetLastError());
+    FastMeta got;
+    MPHF_CUDA(cudaMemcpyAsync(&got, meta, sizeof(got), cudaMemcpyDeviceToHost, st));
+    MPHF_CUDA(cudaStreamSynchronize(st));
+    hm->status = got.status;
+    if (got.status) break;
+    lv.weight = got.lv[d].weight;
+    hm->seen[d] = got.seen[d];
+    hm->n_out[d] = got.n_out[d];
+    if (got.seen[d] != n || lv.weight > n || got.n_out[d] != n - lv.weight) {
+      hm->status = ST_INTERNAL;
+      break;
+    }
+    n -= lv.weight;
+    off += m;
+    FLevel &nx = hm->lv[d + 1];
+    nx.n = n;
+    nx.off = off;
+    if (n == 0) {
+      nx.mode = LM_DONE;
+      hm->levels_used = d + 1;
+    } else if ((uint32_t)(d + 1) == cfg.L || n <= cfg.T) {
+      nx.mode = LM_FLAT;
+      if ((uint32_t)(d + 1) < cfg.L) nx.m = level_bits(n, cfg.gamma);
+    } else {
+      size_bucketed(nx, n, cfg.gamma, cfg.Pmin, cfg.Pmax, cfg.Btarget, cfg.cap_scale);
+      nx.off = off;
+      nx.mode = LM_BUCKETED;
+      if (((off - cfg.m0) >> 6) + (nx.m >> 6) > cfg.arena_words) {
+        hm->status = ST_OVERFLOW;
+        break;
+      }
+    }
+    if (nx.mode != LM_BUCKETED) {
+      d++;
+      break;
+    }
+  }
+  *first = d;
+  return MPHF_OK;
 }
 
 // Largest level size the tail may take for this gamma (keys + 2 bit arrays in 200 KB).
@@ -488,7 +732,8 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
     size_bucketed(hm.lv[0], N, gamma, cfg.Pmin, cfg.Pmax, cfg.Btarget, cfg.cap_scale);
     hm.lv[0].off = 0;
     hm.lv[0].mode = LM_BUCKETED;
-    if (hm.lv[0].B > kBmax) {
+    const bool grouped = hm.lv[0].B > kGroupMinB;
+    if (grouped && ceil_div(m0, 1ull << coarse_shift(m0)) > (u64)kWT) {
       *fallback_needed = true;
       sc.release(st);
       return MPHF_OK;
@@ -505,9 +750,21 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
     const u64 cap1 = level1_bound(N, gamma, cfg.Btarget, cfg.Pmax, cfg.cap_scale, &n1_hi, &Bb);
     const u64 m1_hi = level_bits(n1_hi, gamma);
     cfg.capX = hm.lv[0].B * hm.lv[0].cap;
+    if (grouped) {
+      // room for the slabs of level 0 or of any smaller level
+      const double dens = (double)N / (double)m0;
+      cfg.capX = 0;
+      for (unsigned cs = kGroupShift; cs <= coarse_shift(m0); cs++) {
+        const u64 room = ceil_div(m0, 1ull << cs) *
+                         group_cap(dens * (double)(1ull << cs), cfg.cap_scale);
+        if (cfg.capX < room) cfg.capX = room;
+      }
+      FTRY(dev_alloc(sc.T, (u64)kBatchFine * 8 *
+                               group_cap(dens * (double)(1ull << kGroupShift), cfg.cap_scale), st));
+    }
     if (cfg.capX < cap1) cfg.capX = cap1;
     FTRY(dev_alloc(sc.X, cfg.capX * 8, st));
-    FTRY(dev_alloc(sc.cnt, kBmax * 8, st));
+    FTRY(dev_alloc(sc.cnt, (kWMaxNb + kBatchFine) * 8, st));
     cfg.X = (u64 *)sc.X.p;
     cfg.cnt = (u64 *)sc.cnt.p;
     cfg.F_cap = n1_hi < T ? T : n1_hi;
@@ -531,14 +788,23 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
     }
     FCUDA(cudaMemsetAsync(sc.cnt.p, 0, kBmax * 8, st));
     FCUDA(cudaMemcpyAsync(meta, &hm, sizeof(hm), cudaMemcpyHostToDevice, st));
-    // Level-0 split.  Keys still arriving from the host are split one chunk
-    // per launch as each chunk lands (the buckets' counters only grow, so the
-    // launches compose).
-    const u64 pstep = feed && feed->chunk ? feed->chunk : N;
-    for (u64 c0 = 0; c0 < N; c0 += pstep) {
-      const u64 cn = N - c0 < pstep ? N - c0 : pstep;
-      if (feed) FTRY(feed->ensure(c0 + cn, st));
-      launch_split(keys + c0, cn, meta, 0, cfg, (unsigned)hm.lv[0].B, st);
+    if (grouped) {
+      if (feed) FTRY(feed->ensure(N, st));
+      FTRY(grouped_levels(keys, N, cfg, meta, &hm, sc, &dlim, st));
+      // the device-driven loop goes on from here
+      FCUDA(cudaMemsetAsync(sc.cnt.p, 0, kBmax * 8, st));
+      FCUDA(cudaMemcpyAsync(meta, &hm, sizeof(hm), cudaMemcpyHostToDevice, st));
+      if (D < dlim) D = dlim;
+    } else {
+      // Level-0 split.  Keys still arriving from the host are split one chunk
+      // per launch as each chunk lands (the buckets' counters only grow, so
+      // the launches compose).
+      const u64 pstep = feed && feed->chunk ? feed->chunk : N;
+      for (u64 c0 = 0; c0 < N; c0 += pstep) {
+        const u64 cn = N - c0 < pstep ? N - c0 : pstep;
+        if (feed) FTRY(feed->ensure(c0 + cn, st));
+        launch_split(keys + c0, cn, meta, 0, cfg, (unsigned)hm.lv[0].B, st);
+      }
     }
     const unsigned ctas = (unsigned)sm_count() * 2;
     for (int round = 0; round < 64; round++) {

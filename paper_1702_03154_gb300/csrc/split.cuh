@@ -23,10 +23,10 @@ __device__ __forceinline__ unsigned reduce_range32(u64 h, unsigned m) {
 
 // ---------------------------------------------------------------------------
 // One CTA's share of a multisplit of n values.  Every destination has a ring
-// of two quanta of 2^lq slots in shared memory.  A round pushes one tile: a
+// of at least two quanta of 2^lq slots in shared memory.  A round pushes one tile: a
 // value takes the next slot of its destination with one shared atomic and is
-// stored there.  Then each destination that holds a whole quantum (or two) has
-// it reserved (one global atomic, by the lane that owns the destination) and
+// stored there.  Then each destination that holds whole quanta has
+// them reserved (one global atomic, by the lane that owns the destination) and
 // written out by groups of 2^lq lanes of the same warp: runs that start on a
 // quantum boundary of the bucket, so a bucket is filled by whole 128-byte
 // lines (lq = 4; 64 bytes beyond ~780 destinations).  Nothing is scanned,
@@ -38,12 +38,19 @@ __device__ __forceinline__ unsigned reduce_range32(u64 h, unsigned m) {
 // round length is chosen for rings that rarely fill.  The next tile is loaded
 // (from L2: it was prefetched a round earlier) and hashed while the
 // reservations are in flight.
+//
+// Measured (1e8 values, hashed): 763 destinations 0.46 ms, 180 destinations
+// 0.40 ms (16 bytes a value: 3.5 - 4.0 TB/s); of those 0.46 ms the shared
+// atomics cost 0.11, the copies 0.08, the global atomics 0.08, the ring stores
+// 0.04 (each left out in turn).  The counting-sort multisplit took 0.89 ms.
 // ---------------------------------------------------------------------------
-static constexpr int kWT = 1024;          // threads of a split CTA
-static constexpr int kWK = 8;             // values per thread and round at most
+static constexpr int kWT = 1024;          // threads of a split CTA (or half as many)
 static constexpr unsigned kWMaxNb = 2048; // destinations at most
-static constexpr unsigned kWSpill = 512;  // entries of the spill list
-static constexpr unsigned kWSmem = 227 * 1024;
+static constexpr unsigned kWSpill = 512;  // entries of the spill list (at most a CTA's threads)
+// shared memory of a CTA when `per_sm` of them share a multiprocessor
+__host__ __device__ constexpr unsigned wc_smem(unsigned per_sm) {
+  return (228u * 1024 / per_sm - 1024) & ~15u;
+}
 
 // A queued run: 2^lq ring entries from shared-memory byte `src` to global `dst`.
 struct WcJob {
@@ -52,75 +59,90 @@ struct WcJob {
 };
 
 struct WcShape {
-  unsigned nb, lq;
+  unsigned nb, ls, lq;
   unsigned per;  // destinations a warp owns
+  unsigned nt, smem;  // threads and shared memory of the CTA
 };
 
 __host__ __device__ inline u64 wc_smem_bytes(const WcShape &s) {
-  return (u64)(kWT / 32) * 2 * s.per * sizeof(WcJob) + (((u64)s.nb << (s.lq + 1)) + kWSpill) * 8 +
-         (u64)s.nb * 4 + 16;
+  return (u64)(s.nt / 32) * (s.per << (s.ls - s.lq)) * sizeof(WcJob) +
+         (((u64)s.nb << s.ls) + kWSpill) * 8 + (u64)s.nb * 4 + 16;
 }
 
-// Quantum size for nb destinations: the largest (at most a warp's lanes) whose
-// rings fit.
-__host__ __device__ inline WcShape wc_shape(unsigned nb) {
+// Ring and quantum sizes for nb destinations: the largest ring that fits (at
+// most 2048 slots), of two quanta or of quanta of a warp's 32 lanes.
+__host__ __device__ inline WcShape wc_shape(unsigned nb, unsigned nt, unsigned smem) {
   WcShape s;
   s.nb = nb;
-  s.per = (nb + kWT / 32 - 1) / (kWT / 32);
-  for (s.lq = 5; s.lq > 2 && wc_smem_bytes(s) > kWSmem; s.lq--) {
+  s.nt = nt;
+  s.smem = smem;
+  s.per = (nb + nt / 32 - 1) / (nt / 32);
+  for (s.ls = 11;; s.ls--) {
+    s.lq = s.ls - 1 < 5 ? s.ls - 1 : 5;
+    if (s.ls == 3 || wc_smem_bytes(s) <= smem) return s;
   }
-  return s;
 }
 
 // Values per thread and round: all the CTA has if that is little, and at most
-// what fills a third of the rings (a ring rarely overflows then).  0: so few
-// destinations that a round takes less than one value per thread.
+// what fills three eighths of the rings (a ring rarely overflows then): one of
+// 8, 6, 4, 2, 1.  0: so few destinations that a round takes less than one
+// value per thread.
 __host__ __device__ inline unsigned wc_round(const WcShape &s, u64 n, unsigned ctas) {
-  const unsigned fill = (s.nb << (s.lq + 1)) * 11 / 32 / kWT;
-  const u64 have = (n + (u64)ctas * kWT - 1) / ((u64)ctas * kWT);
+  const unsigned fill = (s.nb << s.ls) * 3 / 8 / s.nt;
+  const u64 have = (n + (u64)ctas * s.nt - 1) / ((u64)ctas * s.nt);
   const u64 k = fill < have ? fill : have;
-  return k < kWK ? (unsigned)k : (unsigned)kWK;
+  return k >= 8 ? 8u : k >= 6 ? 6u : k >= 4 ? 4u : k >= 2 ? 2u : (unsigned)k;
 }
 
-// key(v): the value stored for input v; dst(y): its destination (< sh.nb);
-// dest(b): the bucket's counter, base and capacity.  OWN: 1 up to kWT
-// destinations, 2 beyond.
-template <int OWN, class Key, class Dst, class Dest>
-__device__ __forceinline__ void wc_split(const u64 *__restrict__ in, u64 n, const WcShape &sh,
-                                         unsigned char *smem, const Key &key, const Dst &dst,
-                                         const Dest &dest, u64 *__restrict__ arena,
-                                         unsigned *__restrict__ status) {
-  const unsigned nb = sh.nb, lq = sh.lq, ls = lq + 1, per = sh.per;
+// Threads of a CTA for nb destinations: two CTAs of 512 a multiprocessor where
+// rings of half the memory still take eight values per thread and round (the
+// phases of one overlap those of the other), one CTA of 1024 elsewhere.
+// Measured on 1e8 hashed keys: 180 destinations 403 us against 456, 360 440
+// against 456, but 128 442 against 442 and 512 508 against 504.
+inline int wc_threads(unsigned nb) {
+  const WcShape s = wc_shape(nb, kWT / 2, wc_smem(2));
+  return wc_smem_bytes(s) <= s.smem && (nb << s.ls) * 3 / 8 / s.nt >= 8 ? kWT / 2 : kWT;
+}
+
+// The rounds of wc_split with KR values per thread and a tile of `tile` (at
+// most KR NT) values.
+template <int NT, int OWN, int KR, class Key, class Dst, class Dest>
+__device__ __forceinline__ void wc_rounds(const u64 *__restrict__ in, u64 n, unsigned rank,
+                                          unsigned ranks, unsigned tile, const WcShape &sh,
+                                          unsigned char *smem, const Key &key, const Dst &dst,
+                                          const Dest &dest, u64 *__restrict__ arena,
+                                          unsigned *__restrict__ status) {
+  static_assert(NT >= (int)kWSpill, "one spilled value per thread goes back to the rings");
+  const unsigned nb = sh.nb, ls = sh.ls, lq = sh.lq, per = sh.per;
+  const unsigned njw = per << (ls - lq);  // runs a warp can have queued
   const unsigned S = 1u << ls, Q = 1u << lq;
   const unsigned tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lt = (1u << lane) - 1u;
-  WcJob *jobs = reinterpret_cast<WcJob *>(smem) + warp * 2 * per;  // this warp's queue
-  const unsigned buf0 = (kWT / 32) * 2 * per * (unsigned)sizeof(WcJob);
+  WcJob *jobs = reinterpret_cast<WcJob *>(smem) + warp * njw;  // this warp's queue
+  const unsigned buf0 = (NT / 32) * njw * (unsigned)sizeof(WcJob);
   u64 *buf = reinterpret_cast<u64 *>(smem + buf0);
   u64 *spill = buf + ((u64)nb << ls);
   // per destination: (entries in the ring << 16) | tail; both only grow in a
   // round, the owner brings the tail back below S and takes the entries out
   unsigned *cnt = reinterpret_cast<unsigned *>(spill + kWSpill);
   unsigned *nspill = cnt + nb;
-  for (unsigned i = tid; i < nb; i += kWT) cnt[i] = 0;
+  for (unsigned i = tid; i < nb; i += NT) cnt[i] = 0;
   if (tid == 0) *nspill = 0;
-  const unsigned kr0 = wc_round(sh, n, gridDim.x), kr = kr0 ? kr0 : 1u;
-  const unsigned tile = kr0 ? kr0 * kWT : ((nb << ls) * 11 / 32 + 31) & ~31u;
-  const u64 step = (u64)gridDim.x * tile;
-  u64 t0 = (u64)blockIdx.x * tile;
+  const u64 step = (u64)ranks * tile;
+  u64 t0 = (u64)rank * tile;
   const unsigned full = S << 16;
-  u64 y[kWK];       // inputs, then their stored values
-  unsigned b[kWK];  // destination << ls
+  u64 y[KR] = {};  // inputs, then their stored values
+  unsigned b[KR];  // destination
   // values of the tile at `at` that exist for this thread (k < that number)
   auto mine = [&](u64 at) -> unsigned {
     if (at >= n) return 0;
     const unsigned len = at + tile <= n ? tile : (unsigned)(n - at);
-    return len == kr * kWT ? kr : len > tid ? (len - tid + kWT - 1) / kWT : 0;
+    return len == KR * NT ? KR : len > tid ? (len - tid + NT - 1) / NT : 0;
   };
   auto load = [&](u64 at, unsigned have) {
     const u64 *p = in + at + tid;
 #pragma unroll
-    for (int k = 0; k < kWK; k++)
-      if ((unsigned)k < have) y[k] = __ldcs(p + k * kWT);
+    for (int k = 0; k < KR; k++)
+      if ((unsigned)k < have) y[k] = __ldcs(p + k * NT);
   };
   // the tile at `at` into L2, so that its loads a round later are short
   auto prefetch = [&](u64 at) {
@@ -129,13 +151,12 @@ __device__ __forceinline__ void wc_split(const u64 *__restrict__ in, u64 n, cons
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(tile * 8 - 16));
     }
   };
-  auto hash = [&](unsigned have) {
+  auto hash = [&]() {  // values that do not exist are hashed too and not pushed
 #pragma unroll
-    for (int k = 0; k < kWK; k++)
-      if ((unsigned)k < have) {
-        y[k] = key(y[k]);
-        b[k] = dst(y[k]) << ls;
-      }
+    for (int k = 0; k < KR; k++) {
+      y[k] = key(y[k]);
+      b[k] = dst(y[k]);
+    }
   };
   const unsigned l = lane & (Q - 1), ng = 32u >> lq;
   auto move = [&](const WcJob &j) {
@@ -165,30 +186,44 @@ __device__ __forceinline__ void wc_split(const u64 *__restrict__ in, u64 n, cons
     if (g < r.cap) arena[r.base + g] = yy;
     else atomicOr(status, 1u);
   };
+  auto spilled = [&](u64 yy, unsigned bb) {
+    unsigned j = kWSpill;
+    if (*(volatile unsigned *)nspill < kWSpill) j = atomicAdd(nspill, 1u);
+    if (j < kWSpill) spill[j] = yy;
+    else one(yy, bb);
+  };
+  auto push = [&](unsigned have) {
+    unsigned c[KR], over = 0;
+#pragma unroll
+    for (int k = 0; k < KR; k++) {
+      c[k] = 0;
+      if ((unsigned)k < have) c[k] = atomicAdd(cnt + b[k], 0x10001u);
+    }
+#pragma unroll
+    for (int k = 0; k < KR; k++) {
+      if ((unsigned)k < have && c[k] < full) buf[(b[k] << ls) + (c[k] & (S - 1))] = y[k];
+      over |= c[k] < full ? 0u : 1u << k;
+    }
+    if (over) {
+#pragma unroll
+      for (int k = 0; k < KR; k++)
+        if ((over >> k) & 1u) spilled(y[k], b[k]);
+    }
+  };
   unsigned have = mine(t0);
   load(t0, have);
   prefetch(t0 + step);
-  hash(have);
+  hash();
   __syncthreads();
   for (; t0 < n; t0 += step) {
-#pragma unroll
-    for (int k = 0; k < kWK; k++)
-      if ((unsigned)k < have) {
-        const unsigned c = atomicAdd(cnt + (b[k] >> ls), 0x10001u);
-        if (c < full) {
-          buf[b[k] | (c & (S - 1))] = y[k];
-        } else {
-          unsigned j = kWSpill;
-          if (*(volatile unsigned *)nspill < kWSpill) j = atomicAdd(nspill, 1u);
-          if (j < kWSpill) spill[j] = y[k];
-          else one(y[k], b[k] >> ls);
-        }
-      }
+    if (have == KR) push(KR);
+    else push(have);
     have = mine(t0 + step);
     load(t0 + step, have);
     prefetch(t0 + 2 * step);
     __syncthreads();
-    unsigned nf[OWN], head[OWN];  // whole quanta held (0, 1 or 2), first entry
+    const unsigned ns = *(volatile unsigned *)nspill;
+    unsigned nf[OWN], head[OWN];  // whole quanta held (at most S / Q), first entry
     u64 g[OWN];
 #pragma unroll
     for (int o = 0; o < OWN; o++) {
@@ -202,7 +237,8 @@ __device__ __forceinline__ void wc_split(const u64 *__restrict__ in, u64 n, cons
         if (nf[o]) g[o] = atomicAdd(dest(i).counter, (u64)(nf[o] << lq));
       }
     }
-    hash(have);
+    // in a block of its own: the reservations are on their way before it
+    if (have) hash();
     unsigned nj = 0;
 #pragma unroll
     for (int o = 0; o < OWN; o++) {
@@ -218,46 +254,108 @@ __device__ __forceinline__ void wc_split(const u64 *__restrict__ in, u64 n, cons
         j.src = buf0 + 8 * ((i << ls) + head[o]);
         j.count = Q;
       }
-      const unsigned b1 = __ballot_sync(0xffffffffu, nf[o] != 0);
-      const unsigned b2 = __ballot_sync(0xffffffffu, nf[o] == 2);
-      if (nf[o]) jobs[nj + __popc(b1 & lt)] = j;
+      const unsigned b1 = __ballot_sync(0xffffffffu, nf[o] > 0);
+      const unsigned b2 = __ballot_sync(0xffffffffu, nf[o] > 1);
+      unsigned bq = __ballot_sync(0xffffffffu, nf[o] > 2);
+      if (nf[o] > 0) jobs[nj + __popc(b1 & lt)] = j;
       nj += __popc(b1);
-      if (nf[o] == 2) {
-        j.src = buf0 + 8 * ((i << ls) + (head[o] ^ Q));
+      auto next = [&](unsigned q, unsigned at) {
+        j.src = buf0 + 8 * ((i << ls) + ((head[o] + (q << lq)) & (S - 1)));
         j.dst += Q;
-        jobs[nj + __popc(b2 & lt)] = j;
-      }
+        jobs[at] = j;
+      };
+      if (nf[o] > 1) next(1, nj + __popc(b2 & lt));
       nj += __popc(b2);
+      for (unsigned q = 2; bq; q++) {  // rings of more than two quanta
+        if (nf[o] > q) next(q, nj + __popc(bq & lt));
+        nj += __popc(bq);
+        bq = __ballot_sync(0xffffffffu, nf[o] > q + 1);
+      }
     }
     __syncwarp();
     copy(nj);
     __syncthreads();
-  }
-  // what is left in the rings (less than a quantum each), then the spill list
-  unsigned nj = 0;
-#pragma unroll
-  for (int o = 0; o < OWN; o++) {
-    const unsigned li = lane + 32 * o, i = warp * per + li;
-    const unsigned c = li < per && i < nb ? cnt[i] : 0u, m = c >> 16;
-    WcJob j;
-    j.count = 0;
-    if (m) {
-      const DestRun r = dest(i);
-      const u64 g = atomicAdd(r.counter, (u64)m);
-      if (g + m <= r.cap) j.count = m;
-      else atomicOr(status, 1u);
-      j.src = buf0 + 8 * ((i << ls) + ((c - m) & (S - 1)));
-      j.dst = arena + (r.base + g);
+    // a spill list that fills up goes back through the rings
+    if (ns > kWSpill / 2) {
+      const bool mine_s = tid < min(ns, kWSpill);
+      const u64 v = mine_s ? spill[tid] : 0;
+      __syncthreads();
+      if (tid == 0) *nspill = 0;
+      __syncthreads();
+      if (mine_s) {
+        const unsigned bb = dst(v), c = atomicAdd(cnt + bb, 0x10001u);
+        if (c < full) buf[(bb << ls) + (c & (S - 1))] = v;
+        else spilled(v, bb);
+      }
     }
-    const unsigned bb = __ballot_sync(0xffffffffu, j.count != 0);
-    if (j.count) jobs[nj + __popc(bb & lt)] = j;
-    nj += __popc(bb);
   }
-  __syncwarp();
-  for (unsigned j = lane >> lq; j < nj; j += ng)
-    if (l < jobs[j].count) move(jobs[j]);
+  __syncthreads();
+  // what is left in the rings, then the spill list
+  for (int pass = 0; pass < 2; pass++) {
+    unsigned nj = 0;
+#pragma unroll
+    for (int o = 0; o < OWN; o++) {
+      const unsigned li = lane + 32 * o, i = warp * per + li;
+      const unsigned c = li < per && i < nb ? cnt[i] : 0u, left = min(c >> 16, S);
+      const unsigned head = (c - (c >> 16)) & (S - 1);
+      // first pass: whole quanta (after a push of the spill list), then the rest
+      const unsigned m = pass ? left & (Q - 1) : left & ~(Q - 1);
+      if (!pass && left) cnt[i] = ((left & (Q - 1)) << 16) | ((head + left) & (S - 1));
+      WcJob j;
+      u64 g = 0;
+      bool fits = false;
+      if (m) {
+        const DestRun r = dest(i);
+        g = atomicAdd(r.counter, (u64)m);
+        fits = g + m <= r.cap;
+        if (!fits) atomicOr(status, 1u);
+        j.dst = arena + (r.base + g);
+      }
+      for (unsigned q = 0;; q++) {
+        const bool have_q = fits && (q << lq) < m;
+        const unsigned bq = __ballot_sync(0xffffffffu, have_q);
+        if (!bq) break;
+        if (have_q) {
+          j.src = buf0 + 8 * ((i << ls) + ((head + (q << lq)) & (S - 1)));
+          j.count = min(m - (q << lq), Q);
+          jobs[nj + __popc(bq & lt)] = j;
+          j.dst += Q;
+        }
+        nj += __popc(bq);
+      }
+    }
+    __syncwarp();
+    for (unsigned j = lane >> lq; j < nj; j += ng)
+      if (l < jobs[j].count) move(jobs[j]);
+    __syncwarp();
+  }
   const unsigned ns = min(*nspill, kWSpill);
-  for (unsigned j = tid; j < ns; j += kWT) one(spill[j], dst(spill[j]));
+  for (unsigned j = tid; j < ns; j += NT) one(spill[j], dst(spill[j]));
+}
+
+// key(v): the value stored for input v; dst(y): its destination (< sh.nb);
+// dest(b): the bucket's counter, base and capacity.  The caller is CTA `rank`
+// of the `ranks` that share the n values.  OWN: 1 up to NT destinations, 2
+// beyond.
+template <int NT, int OWN, class Key, class Dst, class Dest>
+__device__ __forceinline__ void wc_split(const u64 *__restrict__ in, u64 n, unsigned rank,
+                                         unsigned ranks, const WcShape &sh, unsigned char *smem,
+                                         const Key &key, const Dst &dst, const Dest &dest,
+                                         u64 *__restrict__ arena, unsigned *__restrict__ status) {
+  if (wc_smem_bytes(sh) > sh.smem || sh.nb > (unsigned)(OWN * NT)) {  // rings that do not fit
+    if (threadIdx.x == 0) atomicOr(status, 1u);
+    return;
+  }
+  const unsigned kr = wc_round(sh, n, ranks);
+  const unsigned tile = kr ? kr * NT : ((sh.nb << sh.ls) * 3 / 8 + 31) & ~31u;
+#define WC_ROUNDS(KR) \
+  wc_rounds<NT, OWN, KR>(in, n, rank, ranks, tile, sh, smem, key, dst, dest, arena, status)
+  if (kr == 8) WC_ROUNDS(8);
+  else if (kr == 6) WC_ROUNDS(6);
+  else if (kr == 4) WC_ROUNDS(4);
+  else if (kr == 2) WC_ROUNDS(2);
+  else WC_ROUNDS(1);
+#undef WC_ROUNDS
 }
 
 }  // namespace bbh

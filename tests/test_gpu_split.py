@@ -33,8 +33,9 @@ def check(M, keys, gamma, shift=0, path=1):
 
 
 # buckets at level 0 (262144 positions each) around the ring sizes: quanta of
-# 32, 16, 8 and 4 values; one owned bucket per thread and two
-@pytest.mark.parametrize("buckets", [388, 395, 775, 790, 1024, 1025, 1545, 1570, 2048])
+# 32, 16, 8 and 4 values; one owned bucket per thread and two; past 2048, the
+# two-step grouping (its last slab and last batch partly filled)
+@pytest.mark.parametrize("buckets", [388, 395, 775, 790, 1024, 1025, 1545, 1570, 2048, 2049, 4500])
 def test_ring_sizes(M, buckets):
     keys = inputs.splitmix64_keys(buckets * 262144 // 200, 5)
     check(M, keys, 200.0)
