@@ -159,6 +159,20 @@ void handle_delete(mphf *h) {
   delete h;
 }
 
+void drop_lookup_desc(mphf *h) {
+  DescBlock *b = h->ldblk;
+  if (!b) return;
+  h->ldesc = nullptr;
+  h->ldblk = nullptr;
+  const bool last = b->refs.fetch_sub(1) == 1;
+  if (h->shared) shared_in_use(h->shared);
+  if (last || !h->shared) cudaDeviceSynchronize();
+  if (last) {
+    dev_free(b->mem, 0);
+    delete b;
+  }
+}
+
 void dev_free(DevBuf &b, cudaStream_t s) {
   if (b.p) cudaFreeAsync(b.p, s);
   b.p = nullptr;
@@ -278,7 +292,7 @@ void mphf_free(mphf_t *h) {
   int prev = 0;
   cudaGetDevice(&prev);
   if (prev != h->device) cudaSetDevice(h->device);
-  if (h->ldesc.p) cudaFree(h->ldesc.p);
+  drop_lookup_desc(h);
   if (h->shared) {
     release_shared(h->shared);
   } else {
@@ -422,10 +436,7 @@ int mphf_set_layout(mphf_t *h, uint32_t sector_bytes_, void *stream) {
     if (prev != h->device) cudaSetDevice(prev);
     return rc;
   }
-  if (h->ldesc.p) {  // multi-lookup descriptor of the old arrays
-    cudaFree(h->ldesc.p);
-    h->ldesc = DevBuf();
-  }
+  drop_lookup_desc(h);  // of the old arrays
   if (h->shared) {
     if (h->n_fb) h->fb = fb;
     else h->fb = DevBuf();

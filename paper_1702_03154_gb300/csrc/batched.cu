@@ -936,13 +936,17 @@ static int ws_get(int i, size_t bytes, cudaStream_t st, void **p) {
 struct mphf_shared {
   bbh::DevBuf arena;
   std::atomic<int> refs{0};
+  std::atomic<bool> in_use{false};  // lookups may be reading it (drop_lookup_desc)
 };
 
 namespace bbh {
 
+void shared_in_use(mphf_shared *sh) { sh->in_use.store(true); }
+
 void release_shared(mphf_shared *sh) {
   if (!sh) return;
   if (sh->refs.fetch_sub(1) == 1) {
+    if (sh->in_use.load()) cudaDeviceSynchronize();
     dev_free(sh->arena, 0);  // stream-ordered on the legacy stream, like a handle's own arrays
     delete sh;
   }

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -213,6 +214,14 @@ int sort_fallback(u64 *keys, u64 n, unsigned int *d_dup_flag, cudaStream_t s);
 struct mphf_shared;  // one device arena shared by the handles of a batched build
 namespace bbh {
 void release_shared(mphf_shared *sh);
+void shared_in_use(mphf_shared *sh);  // its release waits for the device first
+
+// Device descriptors of the functions of one lookup_multi call, in one
+// allocation that lives until the last of those functions is released.
+struct DescBlock {
+  std::atomic<unsigned> refs{0};
+  DevBuf mem;
+};
 }
 
 // The handle.  Host copies of the level metadata plus the device arrays.
@@ -233,7 +242,8 @@ struct mphf {
   int device = 0;
   int path = 0;          // 1 bucketed, 2 unbucketed, 3 batched, 4 loaded, 5 without stored F_d
   mphf_shared *shared = nullptr;  // set: S/SB/fb live in a batched arena
-  bbh::DevBuf ldesc;     // device descriptor for multi-function lookups (made on first use)
+  void *ldesc = nullptr;  // device descriptor for multi-function lookups (made on first use)
+  bbh::DescBlock *ldblk = nullptr;  // the allocation that holds it
   // level tables (last, so that a record can be reset without them): entries
   // past L_used (n: past L_used + 1; s: past L) are never read
   uint64_t n[MPHF_MAX_LEVELS + 1] = {0};
@@ -263,4 +273,8 @@ inline bool narrow_positions(const mphf *h) {
 mphf *handle_new();
 bool handle_new_n(unsigned n, mphf **out, bool zero_tables = true);
 void handle_delete(mphf *h);
+// Give up h's multi-lookup descriptor.  Lookups that may still be reading it
+// or the function are waited for: here, or, for a function whose arrays
+// belong to a batched build, when the last of that build is released.
+void drop_lookup_desc(mphf *h);
 }  // namespace bbh
