@@ -706,6 +706,8 @@ __global__ void __launch_bounds__(kTT, 2) k_bcompact(int d, BCfg c) {
 // threads with ~MAXK * 8 bytes of shared memory, so that several tails share
 // an SM (the tail is a chain of short, barrier-bound levels).  Two shapes are
 // compiled; the autotuner picks one per size class.
+static constexpr size_t kBTailSmem = 112 * 1024;  // two CTAs a multiprocessor
+
 template <int NT, int MAXK>
 __global__ void __launch_bounds__(NT) k_btail(BCfg c, u64 mcap, int dlim) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -732,9 +734,9 @@ __global__ void __launch_bounds__(NT) k_btail(BCfg c, u64 mcap, int dlim) {
     if (threadIdx.x == 0) fail_set(st);
     return;
   }
-  TailSmem sm = carve_tail(smem, mcap, MAXK);
+  TailSmem sm = carve_tail(smem, mcap, c.T, MAXK);
   const u64 *src = st->small ? c.keys + st->key_off : c.flat + st->flat_off;
-  for (unsigned i = threadIdx.x; i < n; i += blockDim.x) sm.keys[i] = src[i];
+  stage_keys<NT, MAXK>(src, (unsigned)n, sm.keys, [](u64 v) { return v; });
   if (threadIdx.x == 0) {
     hist[st->small ? 0 : t].n = n;
     hist[st->small ? 0 : t].off = off;
@@ -968,9 +970,9 @@ static int batched_impl(const u64 *d_keys, const u64 *h_off, unsigned S, double 
   const size_t comp_max = split_smem_bytes((unsigned)kBmax, kTile + kIn) + kPmax / 8;
   u64 mcap = 0;
   u64 T = tune.tail_keys;  // keep a tail's shared memory small enough for several CTAs per SM
-  while (T > 64 && tail_smem_bytes(level_bits(T, gamma), tune.tail_keys) > 96 * 1024) T >>= 1;
+  while (T > 64 && tail_smem_bytes(level_bits(T, gamma), T, tune.tail_keys) > kBTailSmem) T >>= 1;
   mcap = level_bits(T, gamma);
-  const size_t tail_b = tail_smem_bytes(mcap, tune.tail_keys);
+  const size_t tail_b = tail_smem_bytes(mcap, T, tune.tail_keys);
   if (!attr) {
     MPHF_CUDA(cudaFuncSetAttribute(k_bpartition0<true>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -982,11 +984,11 @@ static int batched_impl(const u64 *d_keys, const u64 *h_off, unsigned S, double 
                                    (int)comp_max));
     MPHF_CUDA(cudaFuncSetAttribute(k_bfill, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)(kPmax / 4)));
-    // tail_b <= 96 KB by the choice of T above
+    // tail_b <= kBTailSmem by the choice of T above
     MPHF_CUDA(cudaFuncSetAttribute(k_btail<512, 8192>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   100 * 1024));
+                                   (int)kBTailSmem));
     MPHF_CUDA(cudaFuncSetAttribute(k_btail<256, 4096>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   100 * 1024));
+                                   (int)kBTailSmem));
     attr = true;
   }
   for (unsigned s = 0; s < S; s++) out[s] = nullptr;

@@ -45,6 +45,12 @@ __device__ __forceinline__ u64 reduce_range(u64 h, u64 m) {
   return __umul64hi(h, m);
 }
 
+// reduce_range for m < 2^32.
+__device__ __forceinline__ unsigned reduce_range32(u64 h, unsigned m) {
+  const u64 t = ((u64)(unsigned)h * m) >> 32;
+  return (unsigned)(((u64)(unsigned)(h >> 32) * m + t) >> 32);
+}
+
 // Position of key x in A_d (m_d bits).
 __device__ __forceinline__ u64 level_pos(u64 x, u64 s_d, u64 m_d) {
   return reduce_range(mix64(x ^ s_d), m_d);

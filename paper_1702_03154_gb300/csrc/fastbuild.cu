@@ -418,11 +418,11 @@ k_tail(FastMeta *__restrict__ meta, int dlim, FastCfg cfg, u64 mcap) {
     }
     return;
   }
-  TailSmem sm = carve_tail(smem, mcap);
+  TailSmem sm = carve_tail(smem, mcap, cfg.T);
   // F holds the values of the level before (at t = 0 the caller's keys)
   const u64 s_b = t > 0 ? level_seed(cfg.seed, t - 1) : 0;
-  for (unsigned i = threadIdx.x; i < n; i += kTailThreads)
-    sm.keys[i] = t > 0 ? unmix64(cfg.F[i]) ^ s_b : cfg.F[i];
+  stage_keys<kTailThreads, (int)kTailMaxKeys>(
+      cfg.F, (unsigned)n, sm.keys, [=](u64 v) { return t > 0 ? unmix64(v) ^ s_b : v; });
   __syncthreads();
   unsigned used = cta_levels<kTailThreads, (int)kTailMaxKeys>(
       sm, n, t, lvs[t].off, lvs, cfg.gamma, cfg.L, cfg.seed, cfg.A0,
@@ -484,7 +484,7 @@ static int set_attrs() {
   MPHF_CUDA(cudaFuncSetAttribute(k_gfill<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  1 << (kGroupShift - 2)));
   MPHF_CUDA(cudaFuncSetAttribute(k_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 200 * 1024));
+                                 (int)kTailSmemMax));
   g_attr_set = true;
   return MPHF_OK;
 }
@@ -645,12 +645,13 @@ static int grouped_levels(const u64 *keys, u64 N, const FastCfg &cfg, FastMeta *
   return MPHF_OK;
 }
 
-// Largest level size the tail may take for this gamma (keys + 2 bit arrays in 200 KB).
+// Largest level size the tail may take for this gamma (keys, positions and two
+// bit arrays in shared memory).
 static u64 tail_limit(double gamma, u64 *mcap_out) {
   u64 T = kTailMaxKeys;
   while (T > 64) {
     u64 mc = level_bits(T, gamma);
-    if (tail_smem_bytes(mc) <= 200 * 1024) {
+    if (tail_smem_bytes(mc, T) <= kTailSmemMax) {
       *mcap_out = mc;
       return T;
     }
@@ -725,7 +726,7 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
     FCUDA(cudaMemcpyAsync(meta, &hm, sizeof(hm), cudaMemcpyHostToDevice, st));
     {
       LaunchScope ls("tail", st);
-      k_tail<<<1, kTailThreads, tail_smem_bytes(mcap), st>>>(meta, 0, cfg, mcap);
+      k_tail<<<1, kTailThreads, tail_smem_bytes(mcap, T), st>>>(meta, 0, cfg, mcap);
     }
     FCUDA(cudaGetLastError());
   } else {
@@ -816,7 +817,7 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
       }
       {
         LaunchScope ls("tail", st);
-        k_tail<<<1, kTailThreads, tail_smem_bytes(mcap), st>>>(meta, dlim, cfg, mcap);
+        k_tail<<<1, kTailThreads, tail_smem_bytes(mcap, T), st>>>(meta, dlim, cfg, mcap);
       }
       FCUDA(cudaGetLastError());
       FCUDA(cudaMemcpyAsync(&hm, meta, sizeof(hm), cudaMemcpyDeviceToHost, st));

@@ -100,56 +100,9 @@ __host__ __device__ inline void size_bucketed(FLevel &lv, u64 n, double gamma, u
 // ---------------------------------------------------------------------------
 // Block-wide helpers (kTT threads).
 // ---------------------------------------------------------------------------
-template <int NT>
-__device__ __forceinline__ u64 block_sum(u64 v, u64 *red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  u64 s = 0;
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < NT / 32; i++) s += red[i];
-    red[0] = s;
-  }
-  __syncthreads();
-  s = red[0];
-  __syncthreads();
-  return s;
-}
-
-// Exclusive scan of NT values (one per thread); returns the prefix, *total = sum.
-template <int NT>
-__device__ __forceinline__ unsigned block_scan_u32(unsigned v, unsigned *red, unsigned *total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  __syncthreads();
-  if (lane == 31) red[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    unsigned w = lane < NT / 32 ? red[lane] : 0u;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      unsigned y = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += y;
-    }
-    if (lane < NT / 32) red[lane] = w;
-  }
-  __syncthreads();
-  unsigned before = warp ? red[warp - 1] : 0u;
-  *total = red[NT / 32 - 1];
-  __syncthreads();
-  return before + x - v;
-}
-
-// The same scan with two barriers instead of four, for callers that put a
-// block barrier between one call's reads of red and the next call's writes.
+// Exclusive scan of NT values (one per thread); returns the prefix, *total =
+// sum.  Two barriers; the caller puts a block barrier between one call's reads
+// of red and the next call's writes.
 template <int NT>
 __device__ __forceinline__ unsigned block_scan_u32_fenced(unsigned v, unsigned *red,
                                                           unsigned *total) {
@@ -432,10 +385,11 @@ __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_g
 // ---------------------------------------------------------------------------
 struct TailSmem {
   u64 *keys;      // [kTailMaxKeys]
+  unsigned *pos;  // [T] position of each key at the current level
   unsigned *hit;  // [mcap / 32]
   unsigned *col;
-  unsigned *red;  // [32 + 2]
-  u64 *red64;     // [32]
+  u64 *red64;     // [4]
+  unsigned *red;  // [8]
 };
 
 static __device__ void bitonic_sort_smem(u64 *a, unsigned n) {
@@ -461,124 +415,262 @@ static __device__ void bitonic_sort_smem(u64 *a, unsigned n) {
   }
 }
 
-// Returns the number of levels used.  lvs: level records (n/m/off/weight/mode)
-// of this key set; A0 / arena / m0 locate A_d; fb_out receives the sorted
-// fallback (n_fb keys).  NT threads, at most MAXK keys (MAXK / NT <= 32).
+// dst[i] = f(src[i]), i < n: eight loads of a thread in flight (one at a time,
+// their latency was a third of a 10007-key tail).
+template <int NT, int MAXK, class F>
+static __device__ __forceinline__ void stage_keys(const u64 *__restrict__ src, unsigned n,
+                                                  u64 *__restrict__ dst, const F &f) {
+#pragma unroll 1
+  for (unsigned i0 = threadIdx.x; i0 < n; i0 += 8 * NT) {
+    u64 v[8];
+#pragma unroll
+    for (unsigned u = 0; u < 8; u++) v[u] = i0 + u * NT < n ? src[i0 + u * NT] : 0;
+#pragma unroll
+    for (unsigned u = 0; u < 8; u++)
+      if (i0 + u * NT < n) dst[i0 + u * NT] = f(v[u]);
+  }
+}
+
+// level_bits from gamma as a multiple of 2^-20 (g20 = 2^20 gamma, see below):
+// the double product is then exact, and so is this.
+__device__ __forceinline__ unsigned level_bits20(unsigned n, u64 g20) {
+  const u64 c = (((g20 * n + 0xfffffull) >> 20) + 63) & ~63ull;
+  return c < 64 ? 64u : (unsigned)c;
+}
+
+// Returns the number of levels used.  sm.keys holds the n keys; lvs: level
+// records (n/m/off/weight/mode) of this key set; A0 / arena / m0 locate A_d;
+// fb_out receives the sorted fallback (n_fb keys).  NT threads, at most MAXK
+// keys (MAXK / NT <= 32).
+//
+// A chain of short levels on one CTA, bound by latency and by one SM's issue
+// rate (10007 keys: level 0 takes a third of the time).  A level sets the bits
+// and keeps each key's position, barrier, tests the bits and writes A_d,
+// barrier, moves the survivors to the front in any order (one shared atomic a
+// warp, no scan over the block) and clears the bits, barrier: a level of n
+// keys occupies n / 32 warps only.  The last levels, of at most 128 keys, run
+// in one warp on keys in registers, without barriers.  Level sizes come from
+// integers where gamma is a multiple of 2^-20 (the double arithmetic of
+// level_bits took 900 of a late level's 4300 cycles).
+// 10007 keys, 11 levels: 25 us; with a compaction by block scan and 14
+// barriers a level 46 us.
+static constexpr unsigned kWarpKeys = 128;
+
 template <int NT, int MAXK>
-static __device__ unsigned cta_levels(const TailSmem &sm, u64 n, int d0, u64 off, FLevel *lvs,
+static __device__ unsigned cta_levels(const TailSmem &sm, u64 n64, int d0, u64 off, FLevel *lvs,
                                       double gamma, uint32_t L, u64 seed, u64 *A0, u64 *arena,
                                       u64 m0, u64 arena_words, u64 *fb_out, u64 *n_fb_out,
                                       unsigned *status) {
   static_assert(MAXK % NT == 0 && MAXK / NT <= 32, "keys per thread must fit a 32-bit mask");
+  constexpr unsigned KMAX = (unsigned)(MAXK / NT);
+  const unsigned tid = threadIdx.x, lane = tid & 31;
+  unsigned n = (unsigned)n64;
   int d = d0;
-  for (;;) {
-    if (n == 0) {
-      if (threadIdx.x == 0) lvs[d].mode = LM_DONE;
-      return (unsigned)d;
-    }
-    if ((uint32_t)d == L) {
-      bitonic_sort_smem(sm.keys, (unsigned)n);
-      for (unsigned i = threadIdx.x; i < n; i += blockDim.x) {
-        u64 v = sm.keys[i];
-        fb_out[i] = v;
-        if (i + 1 < n && v == sm.keys[i + 1]) atomicOr(status, ST_DUPLICATE);
-      }
-      if (threadIdx.x == 0) {
-        *n_fb_out = n;
-        lvs[d].mode = LM_FLAT;
-        lvs[d].n = n;
-      }
-      __syncthreads();
-      return L;
-    }
-    const u64 m = level_bits(n, gamma);
-    const u64 s = level_seed(seed, (uint32_t)d);
-    const unsigned mw = (unsigned)(m >> 5);
-    for (unsigned i = threadIdx.x; i < mw; i += blockDim.x) {
-      sm.hit[i] = 0;
-      sm.col[i] = 0;
-    }
-    __syncthreads();
-    for (unsigned i = threadIdx.x; i < n; i += blockDim.x) {
-      const u64 p = level_pos(sm.keys[i], s, m);
-      const unsigned bit = 1u << (p & 31);
-      const unsigned old = atomicOr(sm.hit + (p >> 5), bit);
-      if (old & bit) atomicOr(sm.col + (p >> 5), bit);
-    }
-    __syncthreads();
+  // red64: [0] 2^20 gamma if that is an integer below 2^38 (n < 2^15: the
+  // products stay below 2^53), else 0; [1], [2] seeds of even and odd levels;
+  // [3] size of the level (gamma of the other kind).  red: [0 .. 3] ones and
+  // survivors of even and odd levels; [4], [5] what the last warp leaves.
+  if (tid == 0) {
+    const double g = gamma * 1048576.0;
+    const bool whole = g < 274877906944.0 && (double)(u64)g == g;
+    sm.red64[0] = whole ? (u64)g : 0;
+    sm.red64[1 + (d & 1)] = level_seed(seed, (uint32_t)d);
+    sm.red64[3] = (uint32_t)d < L ? level_bits(n, gamma) : 0;  // a fallback may exceed mcap
+    sm.red[0] = sm.red[1] = sm.red[2] = sm.red[3] = 0;
+  }
+  __syncthreads();
+  const u64 g20 = sm.red64[0];
+  unsigned m = (unsigned)sm.red64[3];
+  for (unsigned i = tid; i < m >> 5; i += NT) sm.hit[i] = sm.col[i] = 0;
+  __syncthreads();
+  auto set = [&](unsigned p) {
+    const unsigned bit = 1u << (p & 31);
+    const unsigned old = atomicOr(sm.hit + (p >> 5), bit);
+    if (old & bit) atomicOr(sm.col + (p >> 5), bit);
+  };
+  auto placed = [&](unsigned p) {
+    return ((sm.hit[p >> 5] & ~sm.col[p >> 5]) >> (p & 31)) & 1u;
+  };
+  // A_d, written by `step` threads from `from`; returns the ones of this one's words
+  auto write_A = [&](unsigned from, unsigned step) -> unsigned {
     u64 *Alev = (d == 0) ? A0 : arena + ((off - m0) >> 6);
     // A_d must fit in the space reserved for the levels after the first
     const bool fits = d == 0 || ((off - m0) >> 6) + (m >> 6) <= arena_words;
-    if (!fits && threadIdx.x == 0) atomicOr(status, ST_OVERFLOW);
-    u64 wsum = 0;
-    for (unsigned w = threadIdx.x; w < (unsigned)(m >> 6); w += blockDim.x) {
-      const u64 a = (u64)(sm.hit[2 * w] & ~sm.col[2 * w]) |
-                    ((u64)(sm.hit[2 * w + 1] & ~sm.col[2 * w + 1]) << 32);
-      if (fits) Alev[w] = a;
-      wsum += __popcll(a);
+    if (!fits && from == 0) atomicOr(status, ST_OVERFLOW);
+    unsigned wsum = 0;
+    for (unsigned w = from; w < m >> 6; w += step) {
+      const uint2 h2 = reinterpret_cast<const uint2 *>(sm.hit)[w];
+      const uint2 c2 = reinterpret_cast<const uint2 *>(sm.col)[w];
+      const unsigned lo = h2.x & ~c2.x, hi = h2.y & ~c2.y;
+      if (fits) Alev[w] = ((u64)hi << 32) | lo;
+      wsum += __popc(lo) + __popc(hi);
     }
-    // compaction in place: each thread keeps its contiguous run of keys in registers
-    constexpr unsigned KMAX = (unsigned)(MAXK / NT);
-    const unsigned per = (unsigned)((n + blockDim.x - 1) / blockDim.x);
-    const unsigned lo = threadIdx.x * per;
-    u64 mine[KMAX];
-    unsigned keepmask = 0, c = 0;
+    return wsum;
+  };
+  auto record = [&](unsigned weight, unsigned rest) {
+    if (weight + rest != n) atomicOr(status, ST_INTERNAL);
+    lvs[d].n = n;
+    lvs[d].m = m;
+    lvs[d].off = off;
+    lvs[d].weight = weight;
+    lvs[d].mode = LM_FLAT;
+    lvs[d + 1].n = rest;
+    lvs[d + 1].off = off + m;
+  };
+  while (n > kWarpKeys && (uint32_t)d < L) {
+    const u64 s = sm.red64[1 + (d & 1)];
+    unsigned *cnt = sm.red + 2 * (d & 1);
+    const unsigned w0 = tid & ~31u;  // the warp's first key of a row of NT keys
+    if (tid == NT - 1) sm.red64[1 + ((d + 1) & 1)] = level_seed(seed, (uint32_t)d + 1);
+#pragma unroll 1
+    for (unsigned k0 = 0; k0 * NT + w0 < n; k0 += 4) {
+      unsigned p[4];
 #pragma unroll
-    for (unsigned k = 0; k < KMAX; k++) {
-      mine[k] = 0;
-      const unsigned i = lo + k;
-      if (k < per && i < n) {
-        const u64 x = sm.keys[i];
-        const u64 p = level_pos(x, s, m);
-        const unsigned bit = 1u << (p & 31);
-        const bool placed = (sm.hit[p >> 5] & ~sm.col[p >> 5]) & bit;
-        if (!placed) {
-          mine[k] = x;
-          keepmask |= 1u << k;
-          c++;
+      for (unsigned u = 0; u < 4; u++)
+        if ((k0 + u) * NT + w0 < n)
+          p[u] = reduce_range32(mix64(sm.keys[(k0 + u) * NT + tid] ^ s), m);
+#pragma unroll
+      for (unsigned u = 0; u < 4; u++)
+        if ((k0 + u) * NT + tid < n) {
+          sm.pos[(k0 + u) * NT + tid] = p[u];
+          set(p[u]);
         }
-      }
-    }
-    unsigned total;
-    unsigned pre = block_scan_u32<NT>(c, sm.red, &total);
-    // every thread has read its keys (block_scan synchronises)
-#pragma unroll
-    for (unsigned k = 0; k < KMAX; k++) {
-      if (keepmask & (1u << k)) sm.keys[pre++] = mine[k];
-    }
-    const u64 wt = block_sum<NT>(wsum, sm.red64);
-    if (threadIdx.x == 0) {
-      if (wt + total != n) atomicOr(status, ST_INTERNAL);
-      lvs[d].n = n;
-      lvs[d].m = m;
-      lvs[d].off = off;
-      lvs[d].weight = wt;
-      lvs[d].mode = LM_FLAT;
-    }
-    n = total;
-    off += m;
-    d++;
-    if (threadIdx.x == 0) {
-      lvs[d].n = n;
-      lvs[d].off = off;
     }
     __syncthreads();
+    unsigned left = 0;
+#pragma unroll 1
+    for (unsigned k0 = 0; k0 * NT + w0 < n; k0 += 4) {
+#pragma unroll
+      for (unsigned u = 0; u < 4; u++)
+        if ((k0 + u) * NT + tid < n && !placed(sm.pos[(k0 + u) * NT + tid])) left |= 1u << (k0 + u);
+    }
+    const unsigned wsum = __reduce_add_sync(0xffffffffu, write_A(tid, NT));
+    u64 mine[KMAX];
+    unsigned at = 0;
+    if (w0 < n) {
+      at = __popc(left);  // survivors of the warp's lanes up to this one
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(0xffffffffu, at, o);
+        if (lane >= (unsigned)o) at += v;
+      }
+      unsigned base = 0;
+      if (lane == 31 && at) base = atomicAdd(cnt + 1, at);
+      at += __shfl_sync(0xffffffffu, base, 31) - __popc(left);
+#pragma unroll
+      for (unsigned k = 0; k < KMAX; k++)
+        if ((left >> k) & 1u) mine[k] = sm.keys[k * NT + tid];
+    }
+    if (lane == 0 && wsum) atomicAdd(cnt, wsum);
+    __syncthreads();
+    const unsigned weight = cnt[0], rest = cnt[1];
+    if (left) {
+#pragma unroll
+      for (unsigned k = 0; k < KMAX; k++)
+        if ((left >> k) & 1u) sm.keys[at++] = mine[k];
+    }
+    for (unsigned i = tid; i < m >> 5; i += NT) sm.hit[i] = sm.col[i] = 0;  // levels shrink
+    if (tid == 0) {
+      record(weight, rest);
+      unsigned *other = sm.red + 2 * ((d + 1) & 1);
+      other[0] = other[1] = 0;
+      if (!g20) sm.red64[3] = level_bits(rest, gamma);
+    }
+    off += m;
+    n = rest;
+    d++;
+    __syncthreads();
+    m = g20 ? level_bits20(n, g20) : (unsigned)sm.red64[3];
   }
+  if (n && (uint32_t)d < L) {  // n <= kWarpKeys: one warp
+    if (tid < 32) {
+      constexpr unsigned kPer = kWarpKeys / 32;
+      u64 x[kPer], s = sm.red64[1 + (d & 1)];
+      unsigned alive = 0;
+      const u64 mixed = mix64(seed);
+#pragma unroll
+      for (unsigned k = 0; k < kPer; k++) {
+        if (k * 32 + lane < n) alive |= 1u << k;
+        x[k] = sm.keys[k * 32 + lane];
+      }
+      while (n && (uint32_t)d < L) {
+        unsigned p[kPer];
+#pragma unroll
+        for (unsigned k = 0; k < kPer; k++) {
+          p[k] = reduce_range32(mix64(x[k] ^ s), m);
+          if ((alive >> k) & 1u) set(p[k]);
+        }
+        s = mix64(mixed + (u64)(d + 1));
+        __syncwarp();
+#pragma unroll
+        for (unsigned k = 0; k < kPer; k++)
+          if (((alive >> k) & 1u) && placed(p[k])) alive &= ~(1u << k);
+        const unsigned weight = __reduce_add_sync(0xffffffffu, write_A(lane, 32));
+        const unsigned rest = __reduce_add_sync(0xffffffffu, __popc(alive));
+        __syncwarp();
+        for (unsigned i = lane; i < m >> 5; i += 32) sm.hit[i] = sm.col[i] = 0;
+        if (lane == 0) record(weight, rest);
+        off += m;
+        n = rest;
+        d++;
+        m = g20 ? level_bits20(n, g20) : (unsigned)level_bits(n, gamma);
+        __syncwarp();
+      }
+      // the keys left for the fallback
+      unsigned at = 0;
+#pragma unroll
+      for (unsigned k = 0; k < kPer; k++) {
+        const unsigned bb = __ballot_sync(0xffffffffu, (alive >> k) & 1u);
+        if ((alive >> k) & 1u) sm.keys[at + __popc(bb & ((1u << lane) - 1u))] = x[k];
+        at += __popc(bb);
+      }
+      if (lane == 0) {
+        sm.red[4] = n;
+        sm.red[5] = (unsigned)d;
+      }
+    }
+    __syncthreads();
+    n = sm.red[4];
+    d = (int)sm.red[5];
+  }
+  if (n == 0) {
+    if (tid == 0) lvs[d].mode = LM_DONE;
+    return (unsigned)d;
+  }
+  // level L: the fallback
+  bitonic_sort_smem(sm.keys, n);
+  for (unsigned i = tid; i < n; i += NT) {
+    u64 v = sm.keys[i];
+    fb_out[i] = v;
+    if (i + 1 < n && v == sm.keys[i + 1]) atomicOr(status, ST_DUPLICATE);
+  }
+  if (tid == 0) {
+    *n_fb_out = n;
+    lvs[d].mode = LM_FLAT;
+    lvs[d].n = n;
+  }
+  __syncthreads();
+  return L;
 }
 
-__device__ __forceinline__ TailSmem carve_tail(unsigned char *smem, u64 mcap,
+// Shared memory of a tail: room for maxk keys (a fallback to be sorted), and
+// for the positions and bits of a level of at most T keys (mcap bits).
+__device__ __forceinline__ TailSmem carve_tail(unsigned char *smem, u64 mcap, u64 T,
                                                u64 maxk = kTailMaxKeys) {
   TailSmem t;
   t.keys = reinterpret_cast<u64 *>(smem);
-  t.hit = reinterpret_cast<unsigned *>(smem + maxk * 8);
+  t.red64 = t.keys + maxk;
+  t.hit = reinterpret_cast<unsigned *>(t.red64 + 4);
   t.col = t.hit + (mcap >> 5);
-  t.red64 = reinterpret_cast<u64 *>(t.col + (mcap >> 5));
-  t.red = reinterpret_cast<unsigned *>(t.red64 + 32);
+  t.pos = t.col + (mcap >> 5);
+  t.red = t.pos + T;
   return t;
 }
 
-static inline size_t tail_smem_bytes(u64 mcap, u64 maxk = kTailMaxKeys) {
-  return maxk * 8 + 2 * (mcap >> 5) * 4 + 32 * 8 + 40 * 4;
+static constexpr size_t kTailSmemMax = 226 * 1024;  // of the plain build's tail
+
+static inline size_t tail_smem_bytes(u64 mcap, u64 T, u64 maxk = kTailMaxKeys) {
+  return maxk * 8 + 2 * (mcap >> 5) * 4 + T * 4 + 4 * 8 + 8 * 4;
 }
 
 

@@ -15,12 +15,6 @@ __host__ __device__ __forceinline__ u64 unmix64(u64 z) {
   return z ^ (z >> 30) ^ (z >> 60);
 }
 
-// reduce_range for m < 2^32.
-__device__ __forceinline__ unsigned reduce_range32(u64 h, unsigned m) {
-  const u64 t = ((u64)(unsigned)h * m) >> 32;
-  return (unsigned)(((u64)(unsigned)(h >> 32) * m + t) >> 32);
-}
-
 // ---------------------------------------------------------------------------
 // One CTA's share of a multisplit of n values.  Every destination has a ring
 // of at least two quanta of 2^lq slots in shared memory.  A round pushes one tile: a
