@@ -3,15 +3,25 @@
 //
 // A key needs e^{1/gamma} level probes on average but up to L; a warp that
 // kept 32 keys in lock-step would idle most lanes while its slowest key walks
-// down the levels.  Instead every lane owns kSlots independent query slots,
-// each with its own (key, output index, level).  Each round every active slot
+// down the levels.  Instead every lane owns two independent query slots, each
+// with its own (key, output index, level).  Each round every active slot
 // probes its current level with one load of the record holding its bit (a
 // 256-bit sector or an 8-byte unit, sector.cuh: the A word and a count of the
 // ones before it come together); a slot whose bit is set finishes its rank
 // from those registers and retires, the others move to the next level, and
-// retired slots are refilled from the warp's stream of input keys.  So lanes
-// stay busy, each lane keeps kSlots independent loads in flight, and a placed
+// retired slots are refilled from the warp's range of input keys.  So lanes
+// stay busy, each lane keeps two independent loads in flight, and a placed
 // key costs one memory request per level probed.
+//
+// What bounds it: the probes' latency and rate at the L2 (about half of the 312
+// G/s that nothing but loads reaches), or HBM's random-access rate beyond it.
+// So nothing else may wait or scatter: a warp's keys arrive in a ring in shared
+// memory by asynchronous copies ahead of the slots, the indices replace them
+// there and leave in input order, a block of 64 at a time, once every key of
+// the block has retired.  Measured: 1e8 queries of a 2e9-key function 3.63 ms
+// (3.94 with each key loaded when its slot is refilled and each index stored
+// when its key retires), 2.3e7 queries at gamma 1 in 64-byte sectors 0.57 ms
+// (0.67), 1e8 queries of a function in L2 1.03 ms (1.03).
 #include <cuda_runtime.h>
 #include <stdlib.h>
 
@@ -48,17 +58,36 @@ __device__ __forceinline__ u64 fallback_index(const LookupArgs &a, u64 x) {
   return MPHF_NOT_FOUND;
 }
 
+static constexpr int kLookupWarps = kLookupThreads / 32;
+// Ring of a warp: keys on their way in, keys in the slots, indices until their
+// block of kBlock keys has retired.  The warp takes keys from all but the
+// block that is still arriving.
+static constexpr unsigned kRing = 512, kBlock = 64, kAhead = kRing - kBlock;
+static constexpr unsigned kFlushAt = 5 * kBlock;  // look for a retired block past this many keys
+
+__device__ __forceinline__ void key_async(u64 *smem_dst, const u64 *gsrc) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void key_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void key_wait() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+
 // kNarrow: every m_d < 2^32 and A short enough that bit g's word index
 // g >> kQShift is below 2^32 (A below 2^36 bits); then a probe's position
 // arithmetic is 32-bit: with off_d a multiple of 64,
 //   g >> kQShift = (off_d >> kQShift) + (p >> kQShift),  g & mask = p & mask.
-template <int kSlots, int W, bool kNarrow>
-__global__ void __launch_bounds__(kLookupThreads)
-k_lookup(const u64 *__restrict__ keys, u64 n, u64 csz, u64 *__restrict__ out, LookupArgs a,
+// Warp w takes the keys [w csz, (w + 1) csz).
+template <int W, bool kNarrow>
+__global__ void __launch_bounds__(kLookupThreads, W == 15 ? 3 : 4)
+k_lookup(const u64 *__restrict__ keys, u64 n, unsigned csz, u64 *__restrict__ out, LookupArgs a,
          LevelTable t) {
   using LW = Lay<W>;
   __shared__ u64 ts[MPHF_MAX_LEVELS], tm[MPHF_MAX_LEVELS], toff[MPHF_MAX_LEVELS];
   __shared__ unsigned tm32[MPHF_MAX_LEVELS], toq[MPHF_MAX_LEVELS];
+  __shared__ u64 rings[kLookupWarps][kRing];
   for (unsigned i = threadIdx.x; i < a.L_used; i += kLookupThreads) {
     ts[i] = t.s[i];
     tm[i] = t.m[i];
@@ -70,94 +99,73 @@ k_lookup(const u64 *__restrict__ keys, u64 n, u64 csz, u64 *__restrict__ out, Lo
 
   const unsigned lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-  const u64 nchunks = (n + csz - 1) / csz;
-  const u64 warp_id = ((u64)blockIdx.x * kLookupThreads + threadIdx.x) >> 5;
-  const u64 nwarps = ((u64)gridDim.x * kLookupThreads) >> 5;
-  u64 chunk = warp_id;
-  u64 cursor = chunk * csz;
-  u64 cend = chunk < nchunks ? min(cursor + csz, n) : cursor;
-  bool more = chunk < nchunks;
-
-  u64 x[kSlots], idx[kSlots];
-  unsigned lvl[kSlots];
-  bool act[kSlots];
+  u64 *ring = rings[threadIdx.x >> 5];
+  const u64 c0 = (((u64)blockIdx.x * kLookupThreads + threadIdx.x) >> 5) * csz;
+  if (c0 >= n) return;
+  const unsigned len = (unsigned)min((u64)csz, n - c0);
+  keys += c0;
+  out += c0;
+  unsigned cur = 0;   // keys taken
+  unsigned base = 0;  // keys whose indices have left the ring
+  // keys [i0, i0 + 64) of the range into the ring
+  auto fetch = [&](unsigned i0) {
 #pragma unroll
-  for (int s = 0; s < kSlots; s++) {
-    act[s] = false;
-    lvl[s] = 0;
-    x[s] = 0;
-    idx[s] = 0;
-  }
-
+    for (unsigned i = i0 + lane; i < i0 + kBlock; i += 32)
+      if (i < len) key_async(ring + (i & (kRing - 1)), keys + i);
+    key_commit();
+  };
+  for (unsigned i = 0; i < min(len, kRing); i += kBlock) fetch(i);
+  key_wait<0>();
+  __syncwarp();
+  u64 x[2] = {0, 0};
+  unsigned idx[2] = {0, 0}, lvl[2] = {0, 0};
+  bool act[2] = {false, false};
   for (;;) {
-    // refill retired slots from the warp's input stream (warp-uniform
-    // control); while the current chunk holds a key for every free slot they
-    // are ranked lane by lane, slot 0 first, and filled in one pass
-    unsigned rk[kSlots], nfree = 0;
+    // refill retired slots, slot 0 first, lane by lane
+    const unsigned avail = min(len, base + kAhead) - cur;
+    const unsigned need0 = __ballot_sync(0xffffffffu, !act[0]);
+    const unsigned need1 = __ballot_sync(0xffffffffu, !act[1]);
+    const unsigned rk[2] = {(unsigned)__popc(need0 & lt),
+                            (unsigned)(__popc(need0) + __popc(need1 & lt))};
 #pragma unroll
-    for (int s = 0; s < kSlots; s++) {
-      const unsigned need = __ballot_sync(0xffffffffu, !act[s]);
-      rk[s] = nfree + __popc(need & lt);
-      nfree += __popc(need);
-    }
-    if (nfree && cend - cursor >= nfree) {
-#pragma unroll
-      for (int s = 0; s < kSlots; s++) {
-        if (!act[s]) {
-          const u64 i = cursor + rk[s];
-          idx[s] = i;
-          x[s] = __ldcs(keys + i);
-          lvl[s] = 0;
-          act[s] = true;
-        }
-      }
-      cursor += nfree;
-    }
-#pragma unroll
-    for (int s = 0; s < kSlots; s++) {
-      unsigned need = __ballot_sync(0xffffffffu, !act[s]);
-      while (need && more) {
-        if (cursor >= cend) {
-          chunk += nwarps;
-          if (chunk >= nchunks) {
-            more = false;
-            break;
-          }
-          cursor = chunk * csz;
-          cend = min(cursor + csz, n);
-        }
-        const u64 avail = cend - cursor;
-        const unsigned r = __popc(need & lt);
-        const bool mine = ((need >> lane) & 1u) && (u64)r < avail;
-        if (mine) {
-          idx[s] = cursor + r;
-          x[s] = __ldcs(keys + cursor + r);
-          lvl[s] = 0;
-          act[s] = true;
-        }
-        const unsigned taken = __ballot_sync(0xffffffffu, mine);
-        need &= ~taken;
-        cursor += __popc(taken);
+    for (int s = 0; s < 2; s++) {
+      if (!act[s] && rk[s] < avail) {
+        idx[s] = cur + rk[s];
+        x[s] = ring[idx[s] & (kRing - 1)];
+        lvl[s] = 0;
+        act[s] = true;
       }
     }
-    bool any = false;
+    cur += min((unsigned)(__popc(need0) + __popc(need1)), avail);
+    // the oldest block leaves once its keys have retired; its place goes to
+    // the keys that follow the ring's
+    if (cur - base >= kFlushAt || cur == len) {
+      const unsigned end = min(base + kBlock, len);
+      const bool old = (act[0] && idx[0] < end) || (act[1] && idx[1] < end);
+      if (!__any_sync(0xffffffffu, old)) {
+        __syncwarp();
 #pragma unroll
-    for (int s = 0; s < kSlots; s++) any |= act[s];
-    if (!__any_sync(0xffffffffu, any)) break;
+        for (unsigned u = 0; u < kBlock; u += 32) {
+          const unsigned i = base + u + lane;
+          if (i < end) __stcs(out + i, ring[i & (kRing - 1)]);
+        }
+        fetch(base + kRing);
+        key_wait<1>();
+        __syncwarp();
+        base = end;
+        if (base == len) break;
+      }
+    }
 
     // one probe per active slot: issue all loads, then resolve
-    typename LW::Pos p[kSlots];
-    typename LW::Data v[kSlots];
+    typename LW::Pos p[2];
+    typename LW::Data v[2];
 #pragma unroll
-    for (int s = 0; s < kSlots; s++) {
+    for (int s = 0; s < 2; s++) {
       if (act[s]) {
         const unsigned d = lvl[s];
         if (kNarrow) {
-          // reduce_range for m < 2^32, kept in 32 bits
-          const u64 h = mix64(x[s] ^ ts[d]);
-          const unsigned m32 = tm32[d];
-          const u64 lo = ((u64)(unsigned)h * m32) >> 32;
-          const unsigned pd = (unsigned)(((u64)(unsigned)(h >> 32) * m32 + lo) >> 32);
+          const unsigned pd = reduce_range32(mix64(x[s] ^ ts[d]), tm32[d]);
           p[s] = LW::pos_q(toq[d] + (pd >> LW::kQShift), pd & ((1u << LW::kQShift) - 1u));
         } else {
           p[s] = LW::pos(toff[d] + level_pos(x[s], ts[d], tm[d]));
@@ -166,14 +174,14 @@ k_lookup(const u64 *__restrict__ keys, u64 n, u64 csz, u64 *__restrict__ out, Lo
       }
     }
 #pragma unroll
-    for (int s = 0; s < kSlots; s++) {
+    for (int s = 0; s < 2; s++) {
       if (act[s]) {
         unsigned w = 0;
         if (LW::hit(v[s], p[s], w)) {
-          __stcs(out + idx[s], LW::rank(v[s], p[s], w, a.SB));
+          ring[idx[s] & (kRing - 1)] = LW::rank(v[s], p[s], w, a.SB);
           act[s] = false;
         } else if (++lvl[s] >= a.L_used) {
-          __stcs(out + idx[s], a.n_fb ? fallback_index(a, x[s]) : MPHF_NOT_FOUND);
+          ring[idx[s] & (kRing - 1)] = a.n_fb ? fallback_index(a, x[s]) : MPHF_NOT_FOUND;
           act[s] = false;
         }
       }
@@ -195,27 +203,20 @@ static void fill_tables(const mphf_t *h, LookupArgs &a, LevelTable &t) {
   }
 }
 
-// Query slots per lane: 2 for every layout.  (8-byte units would leave room
-// for more, but measured on a GB300 3, 4 or 6 slots run slower than 2.)
-static constexpr int kUnitSlots = 2;
-
-template <int SLOTS, int W, bool NARROW>
+template <int W, bool NARROW>
 static int launch_lookup(const u64 *keys, u64 n, u64 *out, const LookupArgs &a,
                          const LevelTable &t, cudaStream_t s) {
-  // one wave of resident CTAs: warps take chunks in a fixed order, so a
-  // second wave would only start after the first has drained
-  static unsigned mb_dev[64] = {0};  // per device
+  static unsigned mb_dev[64] = {0};  // resident CTAs, per device
   unsigned &mb = mb_dev[cur_device()];
-  if (!mb) mb = resident_grid(k_lookup<SLOTS, W, NARROW>, kLookupThreads, 0);
-  const u64 csz = lookup_chunk(n, (u64)mb * (kLookupThreads / 32));
-  const u64 nwarps_needed = (n + csz - 1) / csz;
-  const unsigned per_block = kLookupThreads / 32;
-  u64 grid = (nwarps_needed + per_block - 1) / per_block;
-  if (grid > mb) grid = mb;
-  if (grid < 1) grid = 1;
+  if (!mb) mb = resident_grid(k_lookup<W, NARROW>, kLookupThreads, 0);
+  // one range a resident warp, a multiple of 64 keys (a grid of more than one
+  // wave only past 2^30 keys a warp)
+  const u64 warps = (u64)mb * kLookupWarps;
+  u64 csz = ((n + warps - 1) / warps + 63) & ~63ull;
+  if (csz > 1ull << 30) csz = 1ull << 30;
+  const u64 grid = ((n + csz - 1) / csz + kLookupWarps - 1) / kLookupWarps;
   LaunchScope ls("lookup", s);
-  k_lookup<SLOTS, W, NARROW><<<(unsigned)grid, kLookupThreads, 0, s>>>(keys, n, csz, out, a,
-                                                                       t);
+  k_lookup<W, NARROW><<<(unsigned)grid, kLookupThreads, 0, s>>>(keys, n, (unsigned)csz, out, a, t);
   MPHF_CUDA(cudaGetLastError());
   return MPHF_OK;
 }
@@ -226,13 +227,13 @@ int lookup_impl(const mphf_t *h, const u64 *keys, u64 n, u64 *out, cudaStream_t 
   fill_tables(h, a, t);
   const bool narrow = narrow_positions(h);
   if (h->sw == kSectWordsMini)
-    return narrow ? launch_lookup<2, kSectWordsMini, true>(keys, n, out, a, t, s)
-                  : launch_lookup<2, kSectWordsMini, false>(keys, n, out, a, t, s);
+    return narrow ? launch_lookup<kSectWordsMini, true>(keys, n, out, a, t, s)
+                  : launch_lookup<kSectWordsMini, false>(keys, n, out, a, t, s);
   if (h->sw == kUnitBits)
-    return narrow ? launch_lookup<kUnitSlots, kUnitBits, true>(keys, n, out, a, t, s)
-                  : launch_lookup<kUnitSlots, kUnitBits, false>(keys, n, out, a, t, s);
-  return narrow ? launch_lookup<2, kSectWords, true>(keys, n, out, a, t, s)
-                : launch_lookup<2, kSectWords, false>(keys, n, out, a, t, s);
+    return narrow ? launch_lookup<kUnitBits, true>(keys, n, out, a, t, s)
+                  : launch_lookup<kUnitBits, false>(keys, n, out, a, t, s);
+  return narrow ? launch_lookup<kSectWords, true>(keys, n, out, a, t, s)
+                : launch_lookup<kSectWords, false>(keys, n, out, a, t, s);
 }
 
 }  // namespace bbh
