@@ -125,6 +125,11 @@ struct FillArgs {
   unsigned *status;
 };
 
+static constexpr unsigned kFillStage = 256;  // survivors a warp stages at most
+__host__ __device__ constexpr size_t fill_smem(u64 P) {
+  return (size_t)P / 4 + (size_t)(kTT / 32) * kFillStage * 8;
+}
+
 // Adds the ones of the CTA's buckets and the values found in them to wtot and
 // got (thread 0).
 template <bool NARROW>
@@ -137,6 +142,7 @@ __device__ __forceinline__ void fill_compact(const FillArgs &a, unsigned char *s
   unsigned *hit = reinterpret_cast<unsigned *>(smem);
   unsigned *col = hit + Pw;
   const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
+  u64 *stage = reinterpret_cast<u64 *>(col + Pw) + (threadIdx.x >> 5) * kFillStage;
   for (u64 b = blockIdx.x; b < a.B; b += gridDim.x) {
     for (unsigned i = threadIdx.x; i < Pw / 2; i += kTT)
       reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0, 0, 0, 0);
@@ -147,40 +153,50 @@ __device__ __forceinline__ void fill_compact(const FillArgs &a, unsigned char *s
     const unsigned nv = nk >> 1;  // pairs of values
     auto val0 = [](const uint4 &v) { return ((u64)v.y << 32) | v.x; };
     auto val1 = [](const uint4 &v) { return ((u64)v.w << 32) | v.z; };
+    // position in the bucket; -p0 rides in the upper half of the last product's
+    // addend
+    auto local = [&](u64 y) -> unsigned {
+      if (NARROW) {
+        const unsigned m = (unsigned)a.m;
+        const u64 t = ((u64)(unsigned)y * m) >> 32;
+        return (unsigned)(((u64)(unsigned)(y >> 32) * m + (((u64)(0u - p0) << 32) | t)) >> 32);
+      }
+      return (unsigned)__umul64hi(y, a.m) - p0;
+    };
     __syncthreads();
-    // pass 1: U pairs in flight per thread
-    constexpr int U = 4;
+    constexpr int U = 4;  // pairs in flight per thread
     constexpr unsigned kStep = U * kTT;
-    const unsigned nsteps = (nv + kStep - 1) / kStep;
+    const unsigned nfull = nv / kStep, nsteps = (nv + kStep - 1) / kStep;
     // step s of the bucket into L2 (its loads come later)
     auto ahead = [&](unsigned s) {
       if (threadIdx.x == 0 && s < nsteps)
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(y4 + s * kStep),
                      "r"(min(kStep, nv - s * kStep) * 16));
     };
+    // pass 1
     auto set = [&](u64 y) {
-      const unsigned q = position<NARROW>(y, a.m) - p0;
+      const unsigned q = local(y);
       const unsigned bit = 1u << (q & 31);
       const unsigned old = atomicOr(hit + (q >> 5), bit);
       if (old & bit) atomicOr(col + (q >> 5), bit);
     };
     ahead(1);
-    for (unsigned st = 0; st < nsteps; st++) {
-      const unsigned i0 = st * kStep + threadIdx.x;
+    for (unsigned st = 0; st < nfull; st++) {
       ahead(st + 2);
+      const uint4 *src = y4 + st * kStep + threadIdx.x;
       uint4 v[U];
 #pragma unroll
-      for (int u = 0; u < U; u++) {
-        const unsigned i = i0 + (unsigned)u * kTT;
-        if (i < nv) v[u] = __ldcg(y4 + i);
-      }
+      for (int u = 0; u < U; u++) v[u] = __ldcg(src + u * kTT);
 #pragma unroll
       for (int u = 0; u < U; u++) {
-        if (i0 + (unsigned)u * kTT < nv) {
-          set(val0(v[u]));
-          set(val1(v[u]));
-        }
+        set(val0(v[u]));
+        set(val1(v[u]));
       }
+    }
+    for (unsigned i = nfull * kStep + threadIdx.x; i < nv; i += kTT) {
+      const uint4 v = __ldcg(y4 + i);
+      set(val0(v));
+      set(val1(v));
     }
     if ((nk & 1) && threadIdx.x == 0) set(yb[nk - 1]);
     __syncthreads();
@@ -195,8 +211,7 @@ __device__ __forceinline__ void fill_compact(const FillArgs &a, unsigned char *s
       a.A[w0 + w] = ((u64)k2.y << 32) | k2.x;
       wsum += __popc(k2.x) + __popc(k2.y);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) wsum += __shfl_down_sync(0xffffffffu, wsum, o);
+    wsum = __reduce_add_sync(0xffffffffu, wsum);
     if (lane == 0) red[threadIdx.x >> 5] = wsum;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -215,47 +230,46 @@ __device__ __forceinline__ void fill_compact(const FillArgs &a, unsigned char *s
     __syncthreads();
     u64 *out = a.F + s_base;
     const unsigned room = s_room;
-    // pass 2, last step first (it is the likeliest to be still in L2): a warp
-    // step takes U groups of 32 pairs
-    auto kept = [&](u64 y) {
-      const unsigned q = position<NARROW>(y, a.m) - p0;
-      return !((hit[q >> 5] >> (q & 31)) & 1u);
-    };
-    for (unsigned st = nsteps; st-- > 0;) {
-      const unsigned i0 = st * kStep + threadIdx.x;
-      ahead(st - 2);
-      uint4 v[U];
-#pragma unroll
-      for (int u = 0; u < U; u++) {
-        const unsigned i = i0 + (unsigned)u * kTT;
-        v[u] = i < nv ? __ldcs(y4 + i) : make_uint4(0, 0, 0, 0);
-      }
-      unsigned bal[2 * U], tot = 0, keep = 0;
-#pragma unroll
-      for (int u = 0; u < U; u++) {
-        const bool ok = i0 + (unsigned)u * kTT < nv;
-        const bool k0 = ok && kept(val0(v[u])), k1 = ok && kept(val1(v[u]));
-        keep |= (k0 ? 1u : 0u) << (2 * u) | (k1 ? 1u : 0u) << (2 * u + 1);
-        bal[2 * u] = __ballot_sync(0xffffffffu, k0);
-        bal[2 * u + 1] = __ballot_sync(0xffffffffu, k1);
-        tot += __popc(bal[2 * u]) + __popc(bal[2 * u + 1]);
-      }
+    // pass 2, last step first (it is the likeliest to be still in L2): each
+    // warp packs its survivors in its stage and writes them out as one run
+    unsigned cnt = 0;
+    auto flush = [&]() {
+      __syncwarp();
       unsigned at = 0;
-      if (lane == 0 && tot) at = atomicAdd(&s_count, tot);
+      if (lane == 0) at = atomicAdd(&s_count, cnt);
       at = __shfl_sync(0xffffffffu, at, 0);
-      if (at + tot > room) continue;  // F_{d+1} is full (status raised)
+      if (at + cnt <= room)  // else F_{d+1} is full (status raised)
+        for (unsigned j = lane; j < cnt; j += 32) out[at + j] = stage[j];
+      __syncwarp();
+      cnt = 0;
+    };
+    auto put = [&](bool ok, u64 y) {
+      const unsigned q = local(y) & (unsigned)(a.P - 1);  // in range for a value that is none, too
+      const bool keep = ok && !((hit[q >> 5] >> (q & 31)) & 1u);
+      const unsigned bal = __ballot_sync(0xffffffffu, keep);
+      if (keep) stage[cnt + __popc(bal & lt)] = y;
+      cnt += __popc(bal);
+    };
+    static_assert(kFillStage >= 4 * 32 + 4 * 32, "four puts after a stage that was not flushed");
+    for (unsigned st = nsteps; st-- > 0;) {
+      ahead(st - 2);
+      const unsigned i0 = st * kStep + threadIdx.x;
+      uint4 v[U];
+      const bool all = st < nfull;
 #pragma unroll
-      for (int u = 0; u < U; u++) {
-        if ((keep >> (2 * u)) & 1u) out[at + __popc(bal[2 * u] & lt)] = val0(v[u]);
-        at += __popc(bal[2 * u]);
-        if ((keep >> (2 * u + 1)) & 1u) out[at + __popc(bal[2 * u + 1] & lt)] = val1(v[u]);
-        at += __popc(bal[2 * u + 1]);
+      for (int u = 0; u < U; u++)
+        v[u] = all || i0 + u * kTT < nv ? __ldcs(y4 + i0 + u * kTT) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+      for (int u = 0; u < U; u += 2) {
+        put(all || i0 + u * kTT < nv, val0(v[u]));
+        put(all || i0 + u * kTT < nv, val1(v[u]));
+        put(all || i0 + (u + 1) * kTT < nv, val0(v[u + 1]));
+        put(all || i0 + (u + 1) * kTT < nv, val1(v[u + 1]));
+        if (cnt > kFillStage - 4 * 32) flush();
       }
     }
-    if ((nk & 1) && threadIdx.x == 0 && kept(yb[nk - 1])) {
-      const unsigned at = atomicAdd(&s_count, 1u);
-      if (at < room) out[at] = yb[nk - 1];
-    }
+    if (threadIdx.x < 32 && (nk & 1)) put(lane == 0, yb[nk - 1]);
+    if (cnt) flush();
     __syncthreads();
   }
 }
@@ -469,7 +483,7 @@ static int set_attrs() {
     MPHF_CUDA(cudaFuncSetAttribute(split_fn(v & 1 ? kWMaxNb : 1, (v & 2) != 0),
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wc_smem(1)));
   MPHF_CUDA(cudaFuncSetAttribute(k_fill_compact, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(kPmax / 4)));
+                                 (int)fill_smem(kPmax)));
   for (int v = 0; v < 8; v++) {
     const int nt = v & 4 ? kWT : kWT / 2;
     MPHF_CUDA(cudaFuncSetAttribute(gsplit_fn(nt, v & 1, v & 2),
@@ -480,9 +494,9 @@ static int set_attrs() {
                                    (int)wc_smem(kWT / nt)));
   }
   MPHF_CUDA(cudaFuncSetAttribute(k_gfill<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 1 << (kGroupShift - 2)));
+                                 (int)fill_smem(1ull << kGroupShift)));
   MPHF_CUDA(cudaFuncSetAttribute(k_gfill<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 1 << (kGroupShift - 2)));
+                                 (int)fill_smem(1ull << kGroupShift)));
   MPHF_CUDA(cudaFuncSetAttribute(k_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kTailSmemMax));
   g_attr_set = true;
@@ -599,7 +613,7 @@ static int grouped_levels(const u64 *keys, u64 N, const FastCfg &cfg, FastMeta *
       {
         LaunchScope ls("fill_grouped", st);
         (narrow ? k_gfill<true> : k_gfill<false>)<<<grid_for(a.B, 1, (unsigned)sm_count() * 2), kTT,
-                                                    (size_t)a.P / 4, st>>>(
+                                                    fill_smem(a.P), st>>>(
             a, &meta->lv[d].weight, &meta->seen[d]);
       }
     }
@@ -813,7 +827,7 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
         if (dlim > 0) launch_split(nullptr, n1_hi, meta, dlim, cfg, nb1, st);
         LaunchScope ls("fill_compact", st);
         k_fill_compact<<<dlim == 0 && hm.lv[0].B < ctas ? (unsigned)hm.lv[0].B : ctas, kTT,
-                         (size_t)((dlim == 0 ? hm.lv[0].P : cfg.Pmax) / 4), st>>>(meta, dlim, cfg);
+                         fill_smem(dlim == 0 ? hm.lv[0].P : cfg.Pmax), st>>>(meta, dlim, cfg);
       }
       {
         LaunchScope ls("tail", st);
