@@ -89,6 +89,9 @@ __device__ void finish_level(FastMeta *meta, int d, const FastCfg &cfg) {
   } else if (nn <= cfg.T) {
     nx.mode = LM_FLAT;  // tail
     nx.m = level_bits(nn, cfg.gamma);
+  } else if (nn <= cfg.Tmid && level_bits(nn, cfg.gamma) <= cfg.mmid) {
+    nx.mode = LM_MID;
+    nx.m = level_bits(nn, cfg.gamma);
   } else {
     size_bucketed(nx, nn, cfg.gamma, cfg.Pmin, cfg.Pmax, cfg.Btarget, cfg.cap_scale);
     nx.off = vl[d].off + m;
@@ -390,6 +393,201 @@ __global__ void k_unhash(u64 *__restrict__ F, u64 n, u64 s) {
 }
 
 // ---------------------------------------------------------------------------
+// Levels of at most Tmid keys, down to the tail, in one cooperative launch of
+// one CTA a multiprocessor.  A level of 10^4 to 10^6 keys is bound by latency:
+// two launches of a split and a fill took 20 us whatever its size.  Here each
+// CTA keeps its share of the keys in shared memory, the hit and collision bits
+// are in L2 (64-bit words: bits 0-31 hit, 32-63 collision, so a key costs one
+// atomic and the collided ones a second), and a level is: set the bits, grid
+// barrier, test them, drop the placed keys and write A_d, grid barrier.  The
+// two bit arrays take turns; a level clears the other one behind it.
+// Both sides measured (gamma = 2): build of 2e5 keys 150 us against 225, 1e6 166
+// against 243, 3e6 231 against 330; reach of 1e6 / 3.5e6 keys: build of 3e6 249
+// / 231, of 2e7 strings 1079 / 1061.
+// ---------------------------------------------------------------------------
+static constexpr int kMidThreads = 1024;
+static constexpr unsigned kMidKeys = 24576;  // of a CTA
+static constexpr u64 kMidMax = 3500000;      // keys of a level at most
+static constexpr u64 kMidBits = 1ull << 24;  // bits of a level at most (4 MB of words)
+
+// All CTAs' threads wait here; false after about a second (the status is
+// raised and the launch winds down).
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &round, unsigned *status) {
+  __shared__ int ok;
+  __syncthreads();
+  round++;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(bar, 1u);
+    const unsigned want = round * gridDim.x;
+    int spin = 0;
+    while (*(volatile unsigned *)bar < want && spin < (1 << 22)) {
+      __nanosleep(20);
+      spin++;
+    }
+    ok = spin < (1 << 22);
+    if (!ok) atomicOr(status, ST_TIMEOUT);
+    __threadfence();
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
+__global__ void __launch_bounds__(kMidThreads, 1)
+k_mid(const u64 *__restrict__ keys0, FastMeta *__restrict__ meta, int dlim, FastCfg cfg) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  u64 *keys = reinterpret_cast<u64 *>(smem);
+  __shared__ int t_level;
+  __shared__ unsigned s_cnt, s_ones;
+  __shared__ u64 s_m, s_seed, s_nn, s_at;
+  const unsigned tid = threadIdx.x, lane = tid & 31, lt = (1u << lane) - 1u;
+  if (tid == 0) {
+    int t = -1;
+    if (!*(volatile unsigned *)&meta->status)
+      for (int d = 0; d <= dlim && d < (int)cfg.L; d++)
+        if (meta->lv[d].mode == LM_MID) {
+          t = d;
+          break;
+        }
+    t_level = t;
+  }
+  __syncthreads();
+  // the same decision in every CTA: nothing writes these records before the
+  // first grid barrier
+  int d = t_level;
+  if (d < 0) return;
+  u64 n = meta->lv[d].n, off = meta->lv[d].off, m = meta->lv[d].m;
+  const u64 per = (n + gridDim.x - 1) / gridDim.x;
+  const u64 lo = min(n, per * blockIdx.x);
+  unsigned c = (unsigned)min(per, n - lo);  // this CTA's keys
+  if (d == 0) {
+    stage_keys<kMidThreads, (int)kMidKeys>(keys0 + lo, c, keys, [](u64 v) { return v; });
+  } else {
+    const u64 s_b = level_seed(cfg.seed, d - 1);
+    stage_keys<kMidThreads, (int)kMidKeys>(cfg.F + lo, c, keys,
+                                           [=](u64 v) { return unmix64(v) ^ s_b; });
+  }
+  // words [w0, w1) of a level are this CTA's to clear and to write out
+  auto share = [&](u64 words, u64 &w0, u64 &w1) {
+    const u64 step = (words + gridDim.x - 1) / gridDim.x;
+    w0 = min(words, step * blockIdx.x);
+    w1 = min(words, w0 + step);
+  };
+  u64 w0, w1;
+  share(m >> 6, w0, w1);
+  for (u64 w = w0 + tid; w < w1; w += kMidThreads)
+    reinterpret_cast<ulonglong2 *>(cfg.AC[d & 1])[w] = make_ulonglong2(0, 0);
+  unsigned round = 0;
+  if (tid == 0) s_seed = level_seed(cfg.seed, d);
+  if (!grid_barrier(&meta->bar, round, &meta->status)) return;
+  for (;;) {
+    const u64 s = s_seed;
+    const unsigned m32 = (unsigned)m;
+    u64 *AC = cfg.AC[d & 1];
+    auto at = [&](u64 x) { return reduce_range32(mix64(x ^ s), m32); };
+    constexpr unsigned U = 4;
+    for (unsigned i0 = tid; i0 < c; i0 += U * kMidThreads) {
+      unsigned p[U];
+      u64 old[U];
+#pragma unroll
+      for (unsigned u = 0; u < U; u++) {
+        const unsigned i = i0 + u * kMidThreads;
+        p[u] = i < c ? at(keys[i]) : 0;
+        old[u] = i < c ? atomicOr(AC + (p[u] >> 5), 1ull << (p[u] & 31)) : 0;
+      }
+#pragma unroll
+      for (unsigned u = 0; u < U; u++)
+        if ((old[u] >> (p[u] & 31)) & 1ull) atomicOr(AC + (p[u] >> 5), 1ull << (32 + (p[u] & 31)));
+    }
+    if (tid == 0) s_cnt = s_ones = 0;
+    if (!grid_barrier(&meta->bar, round, &meta->status)) return;
+    // keep the keys whose bit is not a lone hit; a chunk is read before any of
+    // it is written, and what is written lies before what is still to be read
+    for (unsigned i0 = 0; i0 < c; i0 += U * kMidThreads) {
+      u64 x[U];
+      unsigned keep = 0, mine = 0;
+#pragma unroll
+      for (unsigned u = 0; u < U; u++) {
+        const unsigned i = i0 + u * kMidThreads + tid;
+        x[u] = i < c ? keys[i] : 0;
+        const unsigned p = at(x[u]) , b = p & 31;
+        const u64 w = i < c ? __ldcg(AC + (p >> 5)) : 0;
+        if (i < c && !(((w >> b) & 1ull) && !((w >> (32 + b)) & 1ull))) keep |= 1u << u;
+      }
+      mine = __popc(keep);
+      unsigned pre = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(0xffffffffu, pre, o);
+        if (lane >= (unsigned)o) pre += v;
+      }
+      __syncthreads();  // the chunk is read
+      unsigned base = 0;
+      if (lane == 31 && pre) base = atomicAdd(&s_cnt, pre);
+      unsigned to = __shfl_sync(0xffffffffu, base, 31) + pre - mine;
+#pragma unroll
+      for (unsigned u = 0; u < U; u++)
+        if ((keep >> u) & 1u) keys[to++] = x[u];
+      __syncthreads();
+    }
+    // A_d, and the other array cleared
+    u64 *Alev = (d == 0) ? cfg.A0 : cfg.arena + ((off - cfg.m0) >> 6);
+    const bool fits = d == 0 || ((off - cfg.m0) >> 6) + (m >> 6) <= cfg.arena_words;
+    unsigned ones = 0;
+    share(m >> 6, w0, w1);
+    for (u64 w = w0 + tid; w < w1; w += kMidThreads) {
+      const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(AC) + w);
+      const unsigned a0 = v.x & ~v.y, a1 = v.z & ~v.w;
+      if (fits) Alev[w] = ((u64)a1 << 32) | a0;
+      ones += __popc(a0) + __popc(a1);
+      reinterpret_cast<ulonglong2 *>(cfg.AC[(d + 1) & 1])[w] = make_ulonglong2(0, 0);
+    }
+    ones = __reduce_add_sync(0xffffffffu, ones);
+    if (lane == 0 && ones) atomicAdd(&s_ones, ones);
+    __syncthreads();
+    c = s_cnt;
+    if (tid == 0) {
+      if (c) atomicAdd(&meta->n_out[d], (u64)c);
+      if (s_ones) atomicAdd(&meta->lv[d].weight, (u64)s_ones);
+      if (!fits) atomicOr(&meta->status, ST_OVERFLOW);
+    }
+    if (!grid_barrier(&meta->bar, round, &meta->status)) return;
+    if (tid == 0) {
+      const u64 nn = __ldcg(&meta->n_out[d]);
+      s_nn = nn;
+      s_m = nn && (uint32_t)(d + 1) < cfg.L ? level_bits(nn, cfg.gamma) : 0;
+      s_seed = level_seed(cfg.seed, d + 1);
+    }
+    __syncthreads();
+    const u64 nn = s_nn;
+    const bool last = !fits || nn <= cfg.T || (uint32_t)(d + 1) == cfg.L;
+    if (blockIdx.x == 0 && tid == 0) {
+      FLevel &lv = meta->lv[d], &nx = meta->lv[d + 1];
+      if (__ldcg(&lv.weight) + nn != n) atomicOr(&meta->status, ST_INTERNAL);
+      lv.mode = LM_BUCKETED;
+      lv.m = m;
+      nx.n = nn;
+      nx.off = off + m;
+      nx.m = s_m;
+      nx.mode = nn == 0 ? LM_DONE : last ? LM_FLAT : LM_BUCKETED;
+      if (nn == 0) meta->levels_used = d + 1;
+    }
+    off += m;
+    n = nn;
+    m = s_m;
+    d++;
+    if (last) break;
+  }
+  // what is left goes to F as values of the last level, for the tail
+  if (n == 0 || c == 0) return;
+  const u64 s_l = level_seed(cfg.seed, d - 1);
+  if (tid == 0) s_at = atomicAdd(&meta->n_mid, (u64)c);
+  __syncthreads();
+  for (unsigned i = tid; i < c; i += kMidThreads)
+    if (s_at + i < cfg.F_cap) cfg.F[s_at + i] = mix64(keys[i] ^ s_l);
+}
+
+// ---------------------------------------------------------------------------
 // Single-CTA level loop: levels d0.. of a key set of at most kTailMaxKeys keys,
 // keys and bit arrays in shared memory.  Writes A_d words, level metadata and
 // the sorted fallback.
@@ -497,6 +695,8 @@ static int set_attrs() {
                                  (int)fill_smem(1ull << kGroupShift)));
   MPHF_CUDA(cudaFuncSetAttribute(k_gfill<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)fill_smem(1ull << kGroupShift)));
+  MPHF_CUDA(cudaFuncSetAttribute(k_mid, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(kMidKeys * 8)));
   MPHF_CUDA(cudaFuncSetAttribute(k_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kTailSmemMax));
   g_attr_set = true;
@@ -518,10 +718,10 @@ static double expect_next(double n, double gamma) {
 }
 
 struct FastScratch {
-  DevBuf meta, X, cnt, F, A0, arena, T;
+  DevBuf meta, X, cnt, F, A0, arena, T, AC;
   void release(cudaStream_t s) {
     dev_free(meta, s); dev_free(X, s); dev_free(cnt, s); dev_free(F, s);
-    dev_free(A0, s); dev_free(arena, s); dev_free(T, s);
+    dev_free(A0, s); dev_free(arena, s); dev_free(T, s); dev_free(AC, s);
   }
 };
 
@@ -641,6 +841,9 @@ static int grouped_levels(const u64 *keys, u64 N, const FastCfg &cfg, FastMeta *
     } else if ((uint32_t)(d + 1) == cfg.L || n <= cfg.T) {
       nx.mode = LM_FLAT;
       if ((uint32_t)(d + 1) < cfg.L) nx.m = level_bits(n, cfg.gamma);
+    } else if (n <= cfg.Tmid && level_bits(n, cfg.gamma) <= cfg.mmid) {
+      nx.mode = LM_MID;
+      nx.m = level_bits(n, cfg.gamma);
     } else {
       size_bucketed(nx, n, cfg.gamma, cfg.Pmin, cfg.Pmax, cfg.Btarget, cfg.cap_scale);
       nx.off = off;
@@ -673,6 +876,17 @@ static u64 tail_limit(double gamma, u64 *mcap_out) {
   }
   *mcap_out = level_bits(64, gamma);
   return 64;
+}
+
+// k_mid on levels of at most n keys each, found by the device at levels <= dlim.
+static int launch_mid(const u64 *keys, u64 n, FastMeta *meta, int dlim, const FastCfg &cfg,
+                      cudaStream_t st) {
+  LaunchScope ls("mid", st);
+  const unsigned g = (unsigned)sm_count();
+  void *args[] = {(void *)&keys, (void *)&meta, (void *)&dlim, (void *)&cfg};
+  MPHF_CUDA(cudaLaunchCooperativeKernel((const void *)k_mid, dim3(g), dim3(kMidThreads), args,
+                                        (size_t)ceil_div(n, g) * 8, st));
+  return MPHF_OK;
 }
 
 // Returns MPHF_OK with *fallback_needed = false on success; *fallback_needed =
@@ -719,10 +933,22 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
     }                                                   \
   } while (0)
 
+  // k_mid's reach (a shrunken bucket capacity, as tests set, keeps to buckets)
+  if (cfg.cap_scale == 1.0) {
+    cfg.Tmid = std::min(kMidMax, (u64)sm_count() * kMidKeys);
+    cfg.mmid = std::min(level_bits(cfg.Tmid, gamma), kMidBits);
+    if (cfg.Tmid <= T) cfg.Tmid = 0;
+  }
   FTRY(dev_alloc(sc.meta, sizeof(FastMeta), st));
   meta = (FastMeta *)sc.meta.p;
   FTRY(dev_alloc(sc.A0, m0 / 8, st));
   cfg.A0 = (u64 *)sc.A0.p;
+  if (cfg.Tmid && N > T) {
+    const u64 words = std::min(m0, cfg.mmid) / 32;
+    FTRY(dev_alloc(sc.AC, 2 * words * 8, st));
+    cfg.AC[0] = (u64 *)sc.AC.p;
+    cfg.AC[1] = cfg.AC[0] + words;
+  }
   if (N <= T) {
     // the whole function in one CTA
     hm.lv[0].n = N;
@@ -743,6 +969,29 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
       k_tail<<<1, kTailThreads, tail_smem_bytes(mcap, T), st>>>(meta, 0, cfg, mcap);
     }
     FCUDA(cudaGetLastError());
+  } else if (N <= cfg.Tmid && m0 <= cfg.mmid) {
+    // every level in k_mid and the tail
+    hm.lv[0].n = N;
+    hm.lv[0].m = m0;
+    hm.lv[0].mode = LM_MID;
+    cfg.F_cap = N;
+    FTRY(dev_alloc(sc.F, N * 8, st));
+    cfg.F = (u64 *)sc.F.p;
+    u64 n1_hi = 0, Bb = 0;
+    level1_bound(N, gamma, cfg.Btarget, cfg.Pmax, cfg.cap_scale, &n1_hi, &Bb);
+    cfg.arena_words = (u64)(L > 1 ? L - 1 : 1) * (level_bits(n1_hi, gamma) / 64);
+    FTRY(dev_alloc(sc.arena, cfg.arena_words * 8, st));
+    cfg.arena = (u64 *)sc.arena.p;
+    if (feed) FTRY(feed->ensure(N, st));
+    FCUDA(cudaMemcpyAsync(meta, &hm, sizeof(hm), cudaMemcpyHostToDevice, st));
+    FTRY(launch_mid(keys, N, meta, 0, cfg, st));
+    {
+      LaunchScope ls("tail", st);
+      k_tail<<<1, kTailThreads, tail_smem_bytes(mcap, T), st>>>(meta, (int)L, cfg, mcap);
+    }
+    FCUDA(cudaGetLastError());
+    FCUDA(cudaMemcpyAsync(&hm, meta, sizeof(hm), cudaMemcpyDeviceToHost, st));
+    FCUDA(cudaStreamSynchronize(st));
   } else {
     size_bucketed(hm.lv[0], N, gamma, cfg.Pmin, cfg.Pmax, cfg.Btarget, cfg.cap_scale);
     hm.lv[0].off = 0;
@@ -796,7 +1045,11 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
       // predicted number of bucketed levels
       double e = expect_next((double)N, gamma);
       D = 1;
-      while (e > (double)T && D < (int)L) {
+      // (a level within 2% of k_mid's reach may turn out larger)
+      auto mid = [&](double x) {
+        return 1.02 * x <= (double)cfg.Tmid && gamma * 1.02 * x <= (double)cfg.mmid - 64.0;
+      };
+      while (e > (double)T && !mid(e) && D < (int)L) {
         e = expect_next(e, gamma);
         D++;
       }
@@ -829,9 +1082,11 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
         k_fill_compact<<<dlim == 0 && hm.lv[0].B < ctas ? (unsigned)hm.lv[0].B : ctas, kTT,
                          fill_smem(dlim == 0 ? hm.lv[0].P : cfg.Pmax), st>>>(meta, dlim, cfg);
       }
+      if (cfg.Tmid) FTRY(launch_mid(nullptr, cfg.Tmid, meta, dlim, cfg, st));
       {
         LaunchScope ls("tail", st);
-        k_tail<<<1, kTailThreads, tail_smem_bytes(mcap, T), st>>>(meta, dlim, cfg, mcap);
+        k_tail<<<1, kTailThreads, tail_smem_bytes(mcap, T), st>>>(meta, cfg.Tmid ? (int)L : dlim,
+                                                                  cfg, mcap);
       }
       FCUDA(cudaGetLastError());
       FCUDA(cudaMemcpyAsync(&hm, meta, sizeof(hm), cudaMemcpyDeviceToHost, st));

@@ -11,7 +11,8 @@ enum LevelMode : unsigned {
   LM_NONE = 0,
   LM_BUCKETED = 1,  // in position-range buckets
   LM_FLAT = 2,      // contiguous in F (input of the tail, or the fallback if d == L)
-  LM_DONE = 3       // no keys left: the function ends at level d - 1
+  LM_DONE = 3,      // no keys left: the function ends at level d - 1
+  LM_MID = 5        // in F, few enough for the one-launch level loop (k_mid)
 };
 
 // Status bits raised on the device.
@@ -34,12 +35,14 @@ struct FastMeta {
   FLevel lv[MPHF_MAX_LEVELS + 1];
   u64 seen[MPHF_MAX_LEVELS + 1];  // keys found in the buckets of level d (consistency check)
   u64 n_out[MPHF_MAX_LEVELS + 1]; // keys written to F_{d+1} by level d's compaction
+  u64 n_mid;             // keys k_mid has put back into F
   u64 n_fb;              // fallback keys
   u64 rank_total;        // ones of A, from the rank table
   unsigned status;
   unsigned levels_used;
   unsigned tail_done;    // 1 once the level loop has finished; 2 if the fallback is left unsorted
   unsigned dup;          // equal neighbours in a fallback sorted outside the tail
+  unsigned bar;          // arrivals at k_mid's grid barrier
 };
 
 // Build-wide constants of the bucketed path.
@@ -58,6 +61,8 @@ struct FastCfg {
   u64 m0;
   u64 arena_words;
   u64 T;                // levels with at most T keys run in the single-CTA tail
+  u64 Tmid, mmid;       // levels of at most Tmid keys and mmid bits run in k_mid (0: none)
+  u64 *AC[2];           // its hit / collision words (mmid / 32 each), by d & 1
   u64 Pmax, Pmin, Btarget;
   double cap_scale;     // bucket capacity multiplier (1 in production; < 1 only in tests)
 };
