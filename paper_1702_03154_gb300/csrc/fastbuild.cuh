@@ -155,6 +155,7 @@ struct DestRun {
 
 // Plain layout: bucket i at arena[i * cap], counters gcnt[i].
 struct UniformDest {
+  static constexpr bool kShared = false;
   u64 *gcnt;
   u64 cap;
   __device__ __forceinline__ DestRun operator()(unsigned i) const {

@@ -95,7 +95,8 @@ __host__ __device__ inline unsigned wc_round(const WcShape &s, u64 n, unsigned c
 // against 456, but 128 442 against 442 and 512 508 against 504.
 inline int wc_threads(unsigned nb) {
   const WcShape s = wc_shape(nb, kWT / 2, wc_smem(2));
-  return wc_smem_bytes(s) <= s.smem && (nb << s.ls) * 3 / 8 / s.nt >= 8 ? kWT / 2 : kWT;
+  return nb <= (unsigned)kWT / 2 && wc_smem_bytes(s) <= s.smem &&
+                 (nb << s.ls) * 3 / 8 / s.nt >= 8 ? kWT / 2 : kWT;
 }
 
 // The rounds of wc_split with KR values per thread and a tile of `tile` (at
@@ -223,12 +224,32 @@ __device__ __forceinline__ void wc_rounds(const u64 *__restrict__ in, u64 n, uns
     for (int o = 0; o < OWN; o++) {
       const unsigned li = lane + 32 * o, i = warp * per + li;
       nf[o] = 0;
+      if (Dest::kShared) g[o] = 0;
       if (li < per && i < nb) {
         const unsigned c = cnt[i], m = min(c >> 16, S);
         head[o] = (c - (c >> 16)) & (S - 1);
         nf[o] = m >> lq;
         cnt[i] = ((m & (Q - 1)) << 16) | ((head[o] + m) & (S - 1));
-        if (nf[o]) g[o] = atomicAdd(dest(i).counter, (u64)(nf[o] << lq));
+        if (!Dest::kShared && nf[o]) g[o] = atomicAdd(dest(i).counter, (u64)(nf[o] << lq));
+      }
+    }
+    // rings that share a counter: one atomic for those of a warp
+    unsigned before[OWN], lead[OWN];
+    if (Dest::kShared) {
+#pragma unroll
+      for (int o = 0; o < OWN; o++) {
+        const unsigned li = lane + 32 * o, i = warp * per + li;
+        u64 *ctr = li < per && i < nb ? dest(i).counter : nullptr;
+        const unsigned same = __match_any_sync(0xffffffffu, (u64)ctr);
+        unsigned sum = 0;
+        before[o] = 0;
+        for (unsigned bit = 0; bit <= ls - lq; bit++) {
+          const unsigned bb = __ballot_sync(0xffffffffu, (nf[o] >> bit) & 1u) & same;
+          before[o] += __popc(bb & lt) << bit;
+          sum += __popc(bb) << bit;
+        }
+        lead[o] = __ffs(same) - 1;
+        if (lane == lead[o] && sum) g[o] = atomicAdd(ctr, (u64)(sum << lq));
       }
     }
     // in a block of its own: the reservations are on their way before it
@@ -238,6 +259,8 @@ __device__ __forceinline__ void wc_rounds(const u64 *__restrict__ in, u64 n, uns
     for (int o = 0; o < OWN; o++) {
       const unsigned i = warp * per + lane + 32 * o;
       WcJob j;
+      if (Dest::kShared)
+        g[o] = __shfl_sync(0xffffffffu, g[o], lead[o]) + ((u64)before[o] << lq);
       if (nf[o]) {
         const DestRun r = dest(i);
         if (g[o] + (nf[o] << lq) > r.cap) {  // past the bucket's end: dropped
@@ -328,7 +351,8 @@ __device__ __forceinline__ void wc_rounds(const u64 *__restrict__ in, u64 n, uns
 }
 
 // key(v): the value stored for input v; dst(y): its destination (< sh.nb);
-// dest(b): the bucket's counter, base and capacity.  The caller is CTA `rank`
+// dest(b): the bucket's counter, base and capacity (Dest::kShared: destinations
+// next to each other may share them).  The caller is CTA `rank`
 // of the `ranks` that share the n values.  OWN: 1 up to NT destinations, 2
 // beyond.
 template <int NT, int OWN, class Key, class Dst, class Dest>
