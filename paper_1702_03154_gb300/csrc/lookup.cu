@@ -26,6 +26,7 @@
 #include <stdlib.h>
 
 #include "common.cuh"
+#include "keyring.cuh"
 #include "sector.cuh"
 
 namespace bbh {
@@ -59,22 +60,6 @@ __device__ __forceinline__ u64 fallback_index(const LookupArgs &a, u64 x) {
 }
 
 static constexpr int kLookupWarps = kLookupThreads / 32;
-// Ring of a warp: keys on their way in, keys in the slots, indices until their
-// block of kBlock keys has retired.  The warp takes keys from all but the
-// block that is still arriving.
-static constexpr unsigned kRing = 512, kBlock = 64, kAhead = kRing - kBlock;
-static constexpr unsigned kFlushAt = 5 * kBlock;  // look for a retired block past this many keys
-
-__device__ __forceinline__ void key_async(u64 *smem_dst, const u64 *gsrc) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void key_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void key_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
 // kNarrow: every m_d < 2^32 and A short enough that bit g's word index
 // g >> kQShift is below 2^32 (A below 2^36 bits); then a probe's position
 // arithmetic is 32-bit: with off_d a multiple of 64,
@@ -209,14 +194,10 @@ static int launch_lookup(const u64 *keys, u64 n, u64 *out, const LookupArgs &a,
   static unsigned mb_dev[64] = {0};  // resident CTAs, per device
   unsigned &mb = mb_dev[cur_device()];
   if (!mb) mb = resident_grid(k_lookup<W, NARROW>, kLookupThreads, 0);
-  // one range a resident warp, a multiple of 64 keys (a grid of more than one
-  // wave only past 2^30 keys a warp)
-  const u64 warps = (u64)mb * kLookupWarps;
-  u64 csz = ((n + warps - 1) / warps + 63) & ~63ull;
-  if (csz > 1ull << 30) csz = 1ull << 30;
+  const unsigned csz = ring_range(n, (u64)mb * kLookupWarps);
   const u64 grid = ((n + csz - 1) / csz + kLookupWarps - 1) / kLookupWarps;
   LaunchScope ls("lookup", s);
-  k_lookup<W, NARROW><<<(unsigned)grid, kLookupThreads, 0, s>>>(keys, n, (unsigned)csz, out, a, t);
+  k_lookup<W, NARROW><<<(unsigned)grid, kLookupThreads, 0, s>>>(keys, n, csz, out, a, t);
   MPHF_CUDA(cudaGetLastError());
   return MPHF_OK;
 }

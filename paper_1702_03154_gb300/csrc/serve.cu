@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "keyring.cuh"
 #include "parts.cuh"
 #include "sector.cuh"
 
@@ -299,25 +300,37 @@ k_lookup_multi(const ReqDev *__restrict__ reqs, unsigned nreq, u64 total, u64 cs
 
 // Lookups against the K functions of a split, without routing the keys: a
 // refilled slot takes its key's part from the part hash, that part's
-// function, and adds the part's offset to the answer.  Slots and probes as in
-// k_lookup_multi (one index space: the n keys).
+// function, and adds the part's offset to the answer.  Slots, probes and the
+// ring as in k_lookup; warp w takes the keys [w csz, (w + 1) csz).
 template <int W, bool NARROW>
 __global__ void __launch_bounds__(kMultiThreads)
-k_lookup_parts(const u64 *__restrict__ keys, u64 n, u64 csz, u64 *__restrict__ out,
+k_lookup_parts(const u64 *__restrict__ keys, u64 n, unsigned csz, u64 *__restrict__ out,
                const LookupDev *const *__restrict__ fns, const u64 *__restrict__ prefix,
                uint32_t K, u64 sp) {
   using LW = Lay<W>;
+  __shared__ u64 rings[kMultiThreads / 32][kRing];
   const unsigned lane = threadIdx.x & 31;
-  const u64 nchunks = (n + csz - 1) / csz;
-  const u64 nwarps = ((u64)gridDim.x * kMultiThreads) >> 5;
-  u64 chunk = ((u64)blockIdx.x * kMultiThreads + threadIdx.x) >> 5;
-  u64 cursor = chunk * csz;
-  u64 cend = chunk < nchunks ? min(cursor + csz, n) : cursor;
-  bool more = chunk < nchunks;
   const unsigned lt = (1u << lane) - 1u;
-  u64 x[kMultiSlots], idx[kMultiSlots];
+  u64 *ring = rings[threadIdx.x >> 5];
+  const u64 c0 = (((u64)blockIdx.x * kMultiThreads + threadIdx.x) >> 5) * csz;
+  if (c0 >= n) return;
+  const unsigned len = (unsigned)min((u64)csz, n - c0);
+  keys += c0;
+  out += c0;
+  unsigned cur = 0;   // keys taken
+  unsigned base = 0;  // keys whose indices have left the ring
+  auto fetch = [&](unsigned i0) {
+#pragma unroll
+    for (unsigned i = i0 + lane; i < i0 + kBlock; i += 32)
+      if (i < len) key_async(ring + (i & (kRing - 1)), keys + i);
+    key_commit();
+  };
+  for (unsigned i = 0; i < min(len, kRing); i += kBlock) fetch(i);
+  key_wait<0>();
+  __syncwarp();
+  u64 x[kMultiSlots];
   const LookupDev *hd[kMultiSlots];
-  unsigned part[kMultiSlots], lvl[kMultiSlots];
+  unsigned part[kMultiSlots], lvl[kMultiSlots], idx[kMultiSlots];
   bool act[kMultiSlots];
 #pragma unroll
   for (int s = 0; s < kMultiSlots; s++) {
@@ -328,41 +341,43 @@ k_lookup_parts(const u64 *__restrict__ keys, u64 n, u64 csz, u64 *__restrict__ o
     part[s] = 0;
     hd[s] = nullptr;
   }
-  auto take = [&](int s, u64 i) {
-    x[s] = __ldcs(keys + i);
-    idx[s] = i;
-    part[s] = part_index(x[s], sp, K);
-    hd[s] = fns[part[s]];
-    lvl[s] = 0;
-    act[s] = true;
-  };
   for (;;) {
+    const unsigned avail = min(len, base + kAhead) - cur;
+    unsigned nfree = 0;
 #pragma unroll
     for (int s = 0; s < kMultiSlots; s++) {
-      unsigned need = __ballot_sync(0xffffffffu, !act[s]);
-      while (need && more) {
-        if (cursor >= cend) {
-          chunk += nwarps;
-          if (chunk >= nchunks) {
-            more = false;
-            break;
-          }
-          cursor = chunk * csz;
-          cend = min(cursor + csz, n);
-        }
-        const u64 avail = cend - cursor;
-        const unsigned r = __popc(need & lt);
-        const bool mine = ((need >> lane) & 1u) && (u64)r < avail;
-        if (mine) take(s, cursor + r);
-        const unsigned taken = __ballot_sync(0xffffffffu, mine);
-        need &= ~taken;
-        cursor += __popc(taken);
+      const unsigned need = __ballot_sync(0xffffffffu, !act[s]);
+      const unsigned rk = nfree + __popc(need & lt);
+      nfree += __popc(need);
+      if (!act[s] && rk < avail) {
+        idx[s] = cur + rk;
+        x[s] = ring[idx[s] & (kRing - 1)];
+        part[s] = part_index(x[s], sp, K);
+        hd[s] = fns[part[s]];
+        lvl[s] = 0;
+        act[s] = true;
       }
     }
-    bool any = false;
+    cur += min(nfree, avail);
+    if (cur - base >= kFlushAt || cur == len) {
+      const unsigned end = min(base + kBlock, len);
+      bool old = false;
 #pragma unroll
-    for (int s = 0; s < kMultiSlots; s++) any |= act[s];
-    if (!__any_sync(0xffffffffu, any)) break;
+      for (int s = 0; s < kMultiSlots; s++) old |= act[s] && idx[s] < end;
+      if (!__any_sync(0xffffffffu, old)) {
+        __syncwarp();
+#pragma unroll
+        for (unsigned u = 0; u < kBlock; u += 32) {
+          const unsigned i = base + u + lane;
+          if (i < end) __stcs(out + i, ring[i & (kRing - 1)]);
+        }
+        fetch(base + kRing);
+        key_wait<1>();
+        __syncwarp();
+        base = end;
+        if (base == len) break;
+      }
+    }
     typename LW::Pos p[kMultiSlots];
     typename LW::Data v[kMultiSlots];
 #pragma unroll
@@ -371,10 +386,7 @@ k_lookup_parts(const u64 *__restrict__ keys, u64 n, u64 csz, u64 *__restrict__ o
         const unsigned d = lvl[s];
         const LookupDev *h = hd[s];
         if (NARROW) {
-          const u64 hh = mix64(x[s] ^ __ldg(h->s + d));
-          const unsigned m32 = __ldg(h->m32 + d);
-          const u64 lo = ((u64)(unsigned)hh * m32) >> 32;
-          const unsigned pd = (unsigned)(((u64)(unsigned)(hh >> 32) * m32 + lo) >> 32);
+          const unsigned pd = reduce_range32(mix64(x[s] ^ __ldg(h->s + d)), __ldg(h->m32 + d));
           p[s] = LW::pos_q(__ldg(h->oq + d) + (pd >> LW::kQShift),
                            pd & ((1u << LW::kQShift) - 1u));
         } else {
@@ -398,7 +410,7 @@ k_lookup_parts(const u64 *__restrict__ keys, u64 n, u64 csz, u64 *__restrict__ o
           done = true;
         }
         if (done) {
-          __stcs(out + idx[s], r == MPHF_NOT_FOUND ? r : r + __ldg(prefix + part[s]));
+          ring[idx[s] & (kRing - 1)] = r == MPHF_NOT_FOUND ? r : r + __ldg(prefix + part[s]);
           act[s] = false;
         }
       }
@@ -412,11 +424,8 @@ static int launch_parts_wn(const LookupDev *const *d_fns, const u64 *prefix, uin
   static u64 maxb_dev[64] = {0};  // one wave of resident CTAs, per device
   u64 &maxb = maxb_dev[cur_device()];
   if (!maxb) maxb = resident_grid(k_lookup_parts<W, NARROW>, kMultiThreads, 0);
-  const u64 csz = lookup_chunk(n, maxb * (kMultiThreads / 32));
-  const u64 chunks = (n + csz - 1) / csz;
-  u64 grid = (chunks + (kMultiThreads / 32) - 1) / (kMultiThreads / 32);
-  if (grid > maxb) grid = maxb;
-  if (grid < 1) grid = 1;
+  const unsigned csz = ring_range(n, maxb * (kMultiThreads / 32));
+  const u64 grid = ((n + csz - 1) / csz + (kMultiThreads / 32) - 1) / (kMultiThreads / 32);
   LaunchScope ls("lookup_parts", s);
   k_lookup_parts<W, NARROW><<<(unsigned)grid, kMultiThreads, 0, s>>>(keys, n, csz, out, d_fns,
                                                                       prefix, K, sp);
