@@ -890,7 +890,8 @@ static int launch_mid(const u64 *keys, u64 n, FastMeta *meta, int dlim, const Fa
 }
 
 // Returns MPHF_OK with *fallback_needed = false on success; *fallback_needed =
-// true (and nothing allocated) when a device-side bound was exceeded.
+// true (and nothing allocated) when a device-side bound was exceeded, or when
+// there is no room for a grouped level's slabs.
 int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaStream_t st,
                mphf_t *h, bool *fallback_needed, KeyFeed *feed) {
   *fallback_needed = false;
@@ -918,6 +919,9 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
   FastMeta *meta = nullptr;
   int dlim = 0;
   int D = 1;  // levels (from 0) launched before the first look at the device's progress
+  // no room for the slabs of a grouped build: the unbucketed path can do with
+  // less (it leaves the keys in their order), so it is asked
+  bool redo_small = false;
 
 #define FTRY(x)                    \
   do {                             \
@@ -1014,6 +1018,7 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
     const u64 cap1 = level1_bound(N, gamma, cfg.Btarget, cfg.Pmax, cfg.cap_scale, &n1_hi, &Bb);
     const u64 m1_hi = level_bits(n1_hi, gamma);
     cfg.capX = hm.lv[0].B * hm.lv[0].cap;
+    redo_small = grouped;
     if (grouped) {
       // room for the slabs of level 0 or of any smaller level
       const double dens = (double)N / (double)m0;
@@ -1114,6 +1119,7 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
   }
   {
     // handle: level metadata, A = A_0 || arena, rank, fallback
+    redo_small = false;
     const uint32_t used = hm.levels_used;
     if (used < 1 || used > L) {
       rc = MPHF_EINTERNAL;
@@ -1170,6 +1176,10 @@ fail:
   cudaGetLastError();
   sc.release(st);
   cudaStreamSynchronize(st);
+  if (rc == MPHF_ENOMEM && redo_small) {
+    *fallback_needed = true;
+    return MPHF_OK;
+  }
   return rc;
 #undef FTRY
 #undef FCUDA
