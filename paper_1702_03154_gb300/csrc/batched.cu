@@ -174,7 +174,7 @@ __global__ void k_btiles(const u64 *__restrict__ key_off, u64 total, BCfg c,
 }
 
 // Each thread owns kKPT consecutive keys of a tile, staged by asynchronous
-// copies while the previous tile is split (the layout of k_partition0).
+// copies while the previous tile is split.
 template <bool ALIGNED>
 __global__ void __launch_bounds__(kTT, 2)
 k_bpartition0(const u64 *__restrict__ key_off, u64 total, BCfg c) {

@@ -370,8 +370,7 @@ static constexpr size_t split_smem_bytes(unsigned nb_cap, unsigned sorted_cap = 
 }
 
 // ---------------------------------------------------------------------------
-// Level 0: partition the caller's keys into position buckets of A_0; each key
-// is stored with its position inside the bucket, so the fill needs no hash.
+// Asynchronous copies into shared memory.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cp_async8(void *smem_dst, const void *gsrc) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
@@ -383,7 +382,6 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
 
 // ---------------------------------------------------------------------------
 // Single-CTA level loop: levels d0.. of a key set of at most kTailMaxKeys keys,
