@@ -174,6 +174,136 @@ k_lookup(const u64 *__restrict__ keys, u64 n, unsigned csz, u64 *__restrict__ ou
   }
 }
 
+// 8-byte units: each slot loads its next key itself and stores its index when
+// its key retires (no ring).  Their probes are ordinary cached loads that lean
+// on a large L1 for the requests in flight, and the rings' 128 KB of shared
+// memory a multiprocessor leave little of it: 1e8 queries of a function in L2
+// 1.01 ms, 1.52 with the ring.  Warps take chunks of csz keys in a fixed order.
+template <bool kNarrow>
+__global__ void __launch_bounds__(kLookupThreads)
+k_lookup_units(const u64 *__restrict__ keys, u64 n, u64 csz, u64 *__restrict__ out, LookupArgs a,
+               LevelTable t) {
+  using LW = Lay<(int)kUnitBits>;
+  __shared__ u64 ts[MPHF_MAX_LEVELS], tm[MPHF_MAX_LEVELS], toff[MPHF_MAX_LEVELS];
+  __shared__ unsigned tm32[MPHF_MAX_LEVELS], toq[MPHF_MAX_LEVELS];
+  for (unsigned i = threadIdx.x; i < a.L_used; i += kLookupThreads) {
+    ts[i] = t.s[i];
+    tm[i] = t.m[i];
+    toff[i] = t.off[i];
+    tm32[i] = (unsigned)t.m[i];
+    toq[i] = (unsigned)(t.off[i] >> LW::kQShift);
+  }
+  __syncthreads();
+
+  const unsigned lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  const u64 nchunks = (n + csz - 1) / csz;
+  const u64 warp_id = ((u64)blockIdx.x * kLookupThreads + threadIdx.x) >> 5;
+  const u64 nwarps = ((u64)gridDim.x * kLookupThreads) >> 5;
+  u64 chunk = warp_id;
+  u64 cursor = chunk * csz;
+  u64 cend = chunk < nchunks ? min(cursor + csz, n) : cursor;
+  bool more = chunk < nchunks;
+
+  u64 x[2], idx[2];
+  unsigned lvl[2];
+  bool act[2];
+#pragma unroll
+  for (int s = 0; s < 2; s++) {
+    act[s] = false;
+    lvl[s] = 0;
+    x[s] = 0;
+    idx[s] = 0;
+  }
+
+  for (;;) {
+    // refill retired slots from the warp's input stream (warp-uniform
+    // control); while the current chunk holds a key for every free slot they
+    // are ranked lane by lane, slot 0 first, and filled in one pass
+    unsigned rk[2], nfree = 0;
+#pragma unroll
+    for (int s = 0; s < 2; s++) {
+      const unsigned need = __ballot_sync(0xffffffffu, !act[s]);
+      rk[s] = nfree + __popc(need & lt);
+      nfree += __popc(need);
+    }
+    if (nfree && cend - cursor >= nfree) {
+#pragma unroll
+      for (int s = 0; s < 2; s++) {
+        if (!act[s]) {
+          const u64 i = cursor + rk[s];
+          idx[s] = i;
+          x[s] = __ldcs(keys + i);
+          lvl[s] = 0;
+          act[s] = true;
+        }
+      }
+      cursor += nfree;
+    }
+#pragma unroll
+    for (int s = 0; s < 2; s++) {
+      unsigned need = __ballot_sync(0xffffffffu, !act[s]);
+      while (need && more) {
+        if (cursor >= cend) {
+          chunk += nwarps;
+          if (chunk >= nchunks) {
+            more = false;
+            break;
+          }
+          cursor = chunk * csz;
+          cend = min(cursor + csz, n);
+        }
+        const u64 avail = cend - cursor;
+        const unsigned r = __popc(need & lt);
+        const bool mine = ((need >> lane) & 1u) && (u64)r < avail;
+        if (mine) {
+          idx[s] = cursor + r;
+          x[s] = __ldcs(keys + cursor + r);
+          lvl[s] = 0;
+          act[s] = true;
+        }
+        const unsigned taken = __ballot_sync(0xffffffffu, mine);
+        need &= ~taken;
+        cursor += __popc(taken);
+      }
+    }
+    bool any = false;
+#pragma unroll
+    for (int s = 0; s < 2; s++) any |= act[s];
+    if (!__any_sync(0xffffffffu, any)) break;
+
+    // one probe per active slot: issue all loads, then resolve
+    LW::Pos p[2];
+    LW::Data v[2];
+#pragma unroll
+    for (int s = 0; s < 2; s++) {
+      if (act[s]) {
+        const unsigned d = lvl[s];
+        if (kNarrow) {
+          const unsigned pd = reduce_range32(mix64(x[s] ^ ts[d]), tm32[d]);
+          p[s] = LW::pos_q(toq[d] + (pd >> LW::kQShift), pd & ((1u << LW::kQShift) - 1u));
+        } else {
+          p[s] = LW::pos(toff[d] + level_pos(x[s], ts[d], tm[d]));
+        }
+        v[s] = LW::load(a.S, p[s]);
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < 2; s++) {
+      if (act[s]) {
+        unsigned w = 0;
+        if (LW::hit(v[s], p[s], w)) {
+          __stcs(out + idx[s], LW::rank(v[s], p[s], w, a.SB));
+          act[s] = false;
+        } else if (++lvl[s] >= a.L_used) {
+          __stcs(out + idx[s], a.n_fb ? fallback_index(a, x[s]) : MPHF_NOT_FOUND);
+          act[s] = false;
+        }
+      }
+    }
+  }
+}
+
 static void fill_tables(const mphf_t *h, LookupArgs &a, LevelTable &t) {
   a.S = (const unsigned *)h->S.p;
   a.SB = (const u64 *)h->SB.p;
@@ -202,6 +332,23 @@ static int launch_lookup(const u64 *keys, u64 n, u64 *out, const LookupArgs &a,
   return MPHF_OK;
 }
 
+template <bool NARROW>
+static int launch_lookup_units(const u64 *keys, u64 n, u64 *out, const LookupArgs &a,
+                               const LevelTable &t, cudaStream_t s) {
+  // one wave of resident CTAs: a second would only start after the first has
+  // drained
+  static unsigned mb_dev[64] = {0};  // per device
+  unsigned &mb = mb_dev[cur_device()];
+  if (!mb) mb = resident_grid(k_lookup_units<NARROW>, kLookupThreads, 0);
+  const u64 csz = lookup_chunk(n, (u64)mb * kLookupWarps);
+  const u64 grid = ((n + csz - 1) / csz + kLookupWarps - 1) / kLookupWarps;
+  LaunchScope ls("lookup", s);
+  k_lookup_units<NARROW><<<(unsigned)(grid > mb ? mb : grid), kLookupThreads, 0, s>>>(
+      keys, n, csz, out, a, t);
+  MPHF_CUDA(cudaGetLastError());
+  return MPHF_OK;
+}
+
 int lookup_impl(const mphf_t *h, const u64 *keys, u64 n, u64 *out, cudaStream_t s) {
   LookupArgs a;
   LevelTable t;
@@ -211,8 +358,8 @@ int lookup_impl(const mphf_t *h, const u64 *keys, u64 n, u64 *out, cudaStream_t 
     return narrow ? launch_lookup<kSectWordsMini, true>(keys, n, out, a, t, s)
                   : launch_lookup<kSectWordsMini, false>(keys, n, out, a, t, s);
   if (h->sw == kUnitBits)
-    return narrow ? launch_lookup<kUnitBits, true>(keys, n, out, a, t, s)
-                  : launch_lookup<kUnitBits, false>(keys, n, out, a, t, s);
+    return narrow ? launch_lookup_units<true>(keys, n, out, a, t, s)
+                  : launch_lookup_units<false>(keys, n, out, a, t, s);
   return narrow ? launch_lookup<kSectWords, true>(keys, n, out, a, t, s)
                 : launch_lookup<kSectWords, false>(keys, n, out, a, t, s);
 }
