@@ -22,10 +22,11 @@ __device__ __forceinline__ void key_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-// Keys for one range a resident warp: a multiple of 64 (a grid of more than
-// one wave only past 2^30 keys a warp).
+// Keys for one range a resident warp: a multiple of 16, a line of keys, so that
+// a batch of a few hundred keys a warp spreads evenly (a grid of more than one
+// wave only past 2^30 keys a warp).
 inline unsigned ring_range(u64 n, u64 warps) {
-  const u64 csz = ((n + warps - 1) / warps + 63) & ~63ull;
+  const u64 csz = ((n + warps - 1) / warps + 15) & ~15ull;
   return csz > 1ull << 30 ? 1u << 30 : (unsigned)csz;
 }
 
