@@ -252,6 +252,13 @@ def run_reference(args):
 
 
 # -------------------------------------------------------- algorithmic bytes
+# Bucketed path: a level of more than 2048 buckets of 2^18 positions is grouped
+# in two splits (coarse slabs, fine buckets) and filled and compacted in shared
+# memory, a batch of slabs at a time; a level of at most 3.5e6 keys and 2^24
+# bits runs in the one-launch level loop; the levels between take one split and
+# one fill each.
+GROUP_MIN_BITS = 2048 << 18
+MID_KEYS, MID_BITS = 3_500_000, 1 << 24
 # Unbucketed path: a level whose hit/collision array (2 bits a position)
 # exceeds 64 MiB is grouped by slab before its fill (coarse and fine
 # multisplit into fixed-capacity ranges, shared-memory fill and compaction);
@@ -263,8 +270,9 @@ def kernel_bytes(h, name: str, n_queries: int) -> int:
     """Algorithmic DRAM bytes of all launches of one kernel in one build (or
     the step's lookup), from the level sizes: every pass over a level's keys
     reads each key once (8 B) and every pass that moves keys writes each once;
-    A_d is written once (m_d / 8 B).  Moving F_0 into position buckets reads
-    and writes every key; a lookup reads its key and writes its index."""
+    A_d is written once (m_d / 8 B).  A split reads and writes every key of its
+    level, a fill reads them and writes the survivors; a lookup reads its key
+    and writes its index."""
     sizes = h.level_sizes()          # n_0 .. n_last, n_fb
     lv = h.levels()                  # (n_d, m_d, off_d, s_d)
     nd = sizes[:-1]
@@ -272,12 +280,16 @@ def kernel_bytes(h, name: str, n_queries: int) -> int:
     if name == "lookup":
         return 16 * n_queries
     if path == 1:
-        if name == "partition":
-            return 16 * sizes[0]
-        if name == "fill_buckets":
-            return sum(8 * n + m // 8 for (n, m, _, _) in lv)
-        if name == "compact_buckets":
-            return sum(8 * nd[d] + 8 * sizes[d + 1] for d in range(len(nd)))
+        big = [d for d, (n, m, _, _) in enumerate(lv) if m > GROUP_MIN_BITS]
+        one = [d for d, (n, m, _, _) in enumerate(lv)
+               if m <= GROUP_MIN_BITS and not (n <= MID_KEYS and m <= MID_BITS)]
+        if name in ("split_coarse", "split_fine"):
+            return sum(16 * nd[d] for d in big)
+        if name == "split":
+            return sum(16 * nd[d] for d in one)
+        if name in ("fill_grouped", "fill_compact"):
+            return sum(8 * nd[d] + 8 * sizes[d + 1] + lv[d][1] // 8
+                       for d in (big if name == "fill_grouped" else one))
         return 0
     grouped = [d for d, (n, m, _, _) in enumerate(lv) if m // 4 > GROUP_MIN_AC_BYTES]
     if name == "slab_count":
@@ -405,32 +417,25 @@ def kernel_table(h, prof, steps, n_queries):
 # keyed by the kernel and, for the lookup, by where A lives (HBM or L2).
 # `src` lists the source files the kernel is built from and `sha` their SHA-1
 # at capture time: when any of them changes the counters no longer describe
-# the kernel and traffic is null.  Units: a "grouped key-visit" is one key of
-# a level grouped by slab (the unbucketed path's levels past 64 MiB of
-# hit/collision bits); a "query" one looked-up key; a "key" one key of F_0.
+# the kernel and traffic is null.  Units: a "grouped key" is one key of a level
+# grouped in two splits; a "query" one looked-up key.
 _HDR = ["common.cuh", "fastbuild.cuh", "sector.cuh"]
+_GROUPED = {"src": ["fastbuild.cu", "split.cuh"] + _HDR, "sha": "2e064e8e4923", "unit": "grouped key"}
+_LOOKUP = {"src": ["lookup.cu", "keyring.cuh"] + _HDR, "sha": "cbb66b001393", "unit": "query"}
 NCU_TRAFFIC = {
-    "slab_scatter": {"src": ["build.cu"] + _HDR, "sha": "3e970480a42b", "unit": "grouped key-visit",
-                     "bytes_per_unit": 35.19,
-                     "note": "3e8-key capture (level 0 grouped: 24 launches of 4 builds, 42.23 GB "
-                             "over 1.2e9 grouped key-visits), scaled by grouped key-visits"},
-    "fine_fill": {"src": ["build.cu"] + _HDR, "sha": "3e970480a42b", "unit": "grouped key-visit",
-                  "bytes_per_unit": 14.52,
-                  "note": "3e8-key capture (20 launches of 4 builds, 17.43 GB over 1.2e9 "
-                          "grouped key-visits), scaled by grouped key-visits"},
-    "lookup@hbm": {"src": ["lookup.cu"] + _HDR, "sha": "590bc6e40776", "unit": "query",
-                   "bytes_per_unit": 114.8,
-                   "note": "3e8-key function (A 140 MB, above L2), 3e7 random member queries x 4 "
-                           "launches, 13.78 GB"},
-    "lookup@l2": {"src": ["lookup.cu"] + _HDR, "sha": "590bc6e40776", "unit": "query",
-                  "bytes_per_unit": 16.25,
-                  "note": "3e7-key function (A 14 MB, in L2), 3e7 random member queries x 2 "
-                          "launches, 0.975 GB"},
-    "partition": {"src": ["fastbuild.cu"] + _HDR, "sha": "5f73b2a05ed5", "unit": "key",
-                  "bytes_per_unit": 18.21, "note": "3e7-key builds (3 launches, 1.639 GB)"},
-    "compact_buckets": {"src": ["fastbuild.cu"] + _HDR, "sha": "5f73b2a05ed5", "unit": "key",
-                        "bytes_per_unit": 23.34,
-                        "note": "3e7-key builds (3 builds, 26 launches, 2.101 GB), per key of F_0"},
+    "split_coarse": {**_GROUPED, "bytes_per_unit": 15.85,
+                     "note": "4e8-key builds (level 0 grouped: 4 launches, 25.36 GB over 1.6e9 "
+                             "grouped keys)"},
+    "split_fine": {**_GROUPED, "bytes_per_unit": 15.54,
+                   "note": "4e8-key builds (12 launches, 24.87 GB over 1.6e9 grouped keys)"},
+    "fill_grouped": {**_GROUPED, "bytes_per_unit": 15.64,
+                     "note": "4e8-key builds (12 launches, 25.03 GB over 1.6e9 grouped keys)"},
+    "lookup@hbm": {**_LOOKUP, "bytes_per_unit": 136.4,
+                   "note": "4e8-key function (A 188 MB, above L2), 3e7 random member queries x 4 "
+                           "launches, 16.37 GB"},
+    "lookup@l2": {**_LOOKUP, "bytes_per_unit": 14.91,
+                  "note": "3e7-key function (A 14 MB, in L2), 3e7 random member queries x 4 "
+                          "launches, 1.789 GB"},
 }
 L2_BYTES = 126 << 20
 
@@ -439,9 +444,8 @@ def traffic_units(h, name: str, n_queries: int):
     """(key into NCU_TRAFFIC, units one step's launches of `name` process)."""
     if name == "lookup":
         return ("lookup@hbm" if h.device_bytes() > L2_BYTES else "lookup@l2"), n_queries
-    if name in ("slab_scatter", "fine_fill"):
-        lv = h.levels()
-        return name, sum(n for (n, m, _, _) in lv if m // 4 > GROUP_MIN_AC_BYTES)
+    if name in ("split_coarse", "split_fine", "fill_grouped"):
+        return name, sum(n for (n, m, _, _) in h.levels() if m > GROUP_MIN_BITS)
     return name, h.level_sizes()[0]
 
 
