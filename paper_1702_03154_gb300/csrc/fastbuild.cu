@@ -176,7 +176,8 @@ __device__ __forceinline__ void fill_compact(const FillArgs &a, unsigned char *s
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(y4 + s * kStep),
                      "r"(min(kStep, nv - s * kStep) * 16));
     };
-    // pass 1
+    // pass 1: every value lies in this bucket, whatever the input (a split fills
+    // an overflowing bucket to its end), so positions need no mask
     auto set = [&](u64 y) {
       const unsigned q = local(y);
       const unsigned bit = 1u << (q & 31);
@@ -338,11 +339,18 @@ static unsigned coarse_shift(u64 m) {
 // 2.6e8 keys (gamma 2, 1984 buckets): one split 5.3 ms a build, two steps 6.1.
 static constexpr u64 kGroupMinB = kBmax;
 
+// A launch behind an overflow does nothing (the host looks once a level).  One
+// decision for the whole CTA: another one may be raising the status now.
+__device__ __forceinline__ bool raised(const unsigned *status) {
+  return __syncthreads_or(*(const volatile unsigned *)status) != 0;
+}
+
 template <int NT, bool FIRST, bool NARROW>
 __global__ void __launch_bounds__(NT, kWT / NT)
 k_gsplit(const u64 *__restrict__ in, u64 n, u64 m, unsigned cs, u64 s_x, unsigned nb,
          u64 *__restrict__ cnt, u64 cap, u64 *__restrict__ out, unsigned *__restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem[];
+  if (raised(status)) return;
   wc_split<NT, 1>(
       in, n, blockIdx.x, gridDim.x, wc_shape(nb, NT, wc_smem(kWT / NT)), smem,
       [=](u64 v) { return mix64((FIRST ? v : unmix64(v)) ^ s_x); },
@@ -360,6 +368,7 @@ k_fsplit(const u64 *__restrict__ R, const u64 *__restrict__ cnt_c, u64 cap_c, un
          unsigned ns, unsigned nf, u64 m, u64 *__restrict__ cnt_f, u64 cap_f, u64 *__restrict__ T,
          unsigned *__restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem[];
+  if (raised(status)) return;
   const unsigned per = gridDim.x / ns, j = blockIdx.x / per;
   const u64 n = min(cnt_c[s0 + j], cap_c);
   const unsigned f0 = (s0 + j) * nf;  // the slab's first fine bucket
@@ -377,6 +386,7 @@ template <bool NARROW>
 __global__ void __launch_bounds__(kTT, 2)
 k_gfill(FillArgs a, u64 *__restrict__ weight, u64 *__restrict__ seen) {
   extern __shared__ __align__(16) unsigned char smem[];
+  if (raised(a.status)) return;
   u64 wtot = 0, got = 0;
   fill_compact<NARROW>(a, smem, wtot, got);
   if (threadIdx.x == 0) {
