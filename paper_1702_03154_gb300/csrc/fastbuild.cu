@@ -782,9 +782,10 @@ static int grouped_levels(const u64 *keys, u64 N, const FastCfg &cfg, FastMeta *
     const u64 cap_f =
         group_cap((double)n * (double)(1ull << kGroupShift) / (double)m, cfg.cap_scale);
     u64 *cnt_c = (u64 *)sc.cnt.p, *cnt_f = cnt_c + kWMaxNb;
-    if (nc > (unsigned)kWT || nc * cap_c > cfg.capX ||
-        (u64)kBatchFine * cap_f * 8 > sc.T.bytes)
-      return MPHF_EINTERNAL;  // cannot happen: sized for level 0, and levels shrink
+    if (nc > (unsigned)kWT || nc * cap_c > cfg.capX || (u64)kBatchFine * cap_f * 8 > sc.T.bytes) {
+      hm->status = ST_OVERFLOW;  // redone by the unbucketed path, like any bound exceeded
+      break;
+    }
     MPHF_CUDA(cudaMemsetAsync(cnt_c, 0, kWMaxNb * 8, st));
     const bool narrow = (m >> 32) == 0;
     const u64 s_d = level_seed(cfg.seed, d);
@@ -1030,16 +1031,16 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
     cfg.capX = hm.lv[0].B * hm.lv[0].cap;
     redo_small = grouped;
     if (grouped) {
-      // room for the slabs of level 0 or of any smaller level
-      const double dens = (double)N / (double)m0;
+      // room for the slabs of level 0 or of any smaller level.  A level's keys per
+      // position may exceed level 0's (both sizes are rounded up to whole words)
+      // but not 1 / gamma; the one step more is for the rounding of the mean
+      auto slots = [&](unsigned shift) {
+        return group_cap((double)(1ull << shift) / gamma, cfg.cap_scale) + 16;
+      };
       cfg.capX = 0;
-      for (unsigned cs = kGroupShift; cs <= coarse_shift(m0); cs++) {
-        const u64 room = ceil_div(m0, 1ull << cs) *
-                         group_cap(dens * (double)(1ull << cs), cfg.cap_scale);
-        if (cfg.capX < room) cfg.capX = room;
-      }
-      FTRY(dev_alloc(sc.T, (u64)kBatchFine * 8 *
-                               group_cap(dens * (double)(1ull << kGroupShift), cfg.cap_scale), st));
+      for (unsigned cs = kGroupShift; cs <= coarse_shift(m0); cs++)
+        cfg.capX = std::max(cfg.capX, ceil_div(m0, 1ull << cs) * slots(cs));
+      FTRY(dev_alloc(sc.T, (u64)kBatchFine * 8 * slots(kGroupShift), st));
     }
     if (cfg.capX < cap1) cfg.capX = cap1;
     FTRY(dev_alloc(sc.X, cfg.capX * 8, st));
