@@ -79,7 +79,7 @@ int mphf_abi_version(void);
  *   stream  work is issued on this stream; the call returns when it is done.
  *   out     receives the new handle (NULL on error).
  * Errors: MPHF_EINVAL, MPHF_ENOMEM, MPHF_EDUPLICATE (nothing is leaked),
- * MPHF_ECUDA, MPHF_EINTERNAL.
+ * MPHF_ECUDA, MPHF_ETIMEOUT, MPHF_EINTERNAL.
  */
 int mphf_build(const uint64_t *d_keys, uint64_t n, double gamma, uint32_t levels, uint64_t seed,
                void *stream, mphf_t **out);
@@ -184,6 +184,11 @@ int mphf_debug_lookup_wide(int on);
  * filled in shared memory (defaults 27 and 64 MiB); no result changes.
  * shift in [6, 29]; MPHF_EINVAL otherwise. */
 int mphf_debug_slabs(uint32_t shift, uint64_t min_ac_bytes);
+
+/* Test hook for the level loop of mid-sized levels (16K to 3.5M keys): looks at
+ * its grid barrier before a wait gives up and the build returns MPHF_ETIMEOUT
+ * (negative: the default, about a second). */
+int mphf_debug_mid(int polls);
 
 /* Test hook: scales the bucket capacities of mphf_build_batched (default 1;
  * values < 1 make sets overflow and exercise their individual rebuild). */

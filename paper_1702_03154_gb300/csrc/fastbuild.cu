@@ -420,9 +420,13 @@ static constexpr unsigned kMidKeys = 24576;  // of a CTA
 static constexpr u64 kMidMax = 3500000;      // keys of a level at most
 static constexpr u64 kMidBits = 1ull << 24;  // bits of a level at most (4 MB of words)
 
-// All CTAs' threads wait here; false after about a second (the status is
-// raised and the launch winds down).
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &round, unsigned *status) {
+static constexpr unsigned kMidPolls = 1u << 22;
+unsigned g_mid_polls = kMidPolls;
+
+// All CTAs' threads wait here; false after `polls` looks, about a second (the
+// status is raised and the launch winds down).
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &round, unsigned polls,
+                                             unsigned *status) {
   __shared__ int ok;
   __syncthreads();
   round++;
@@ -430,12 +434,12 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &round, uns
     __threadfence();
     atomicAdd(bar, 1u);
     const unsigned want = round * gridDim.x;
-    int spin = 0;
-    while (*(volatile unsigned *)bar < want && spin < (1 << 22)) {
+    unsigned spin = 0;
+    while (*(volatile unsigned *)bar < want && spin < polls) {
       __nanosleep(20);
       spin++;
     }
-    ok = spin < (1 << 22);
+    ok = spin < polls;
     if (!ok) atomicOr(status, ST_TIMEOUT);
     __threadfence();
   }
@@ -450,7 +454,7 @@ k_mid(const u64 *__restrict__ keys0, FastMeta *__restrict__ meta, int dlim, Fast
   __shared__ int t_level;
   __shared__ unsigned s_cnt, s_ones;
   __shared__ u64 s_m, s_seed, s_nn, s_at;
-  const unsigned tid = threadIdx.x, lane = tid & 31, lt = (1u << lane) - 1u;
+  const unsigned tid = threadIdx.x, lane = tid & 31;
   if (tid == 0) {
     int t = -1;
     if (!*(volatile unsigned *)&meta->status)
@@ -489,7 +493,7 @@ k_mid(const u64 *__restrict__ keys0, FastMeta *__restrict__ meta, int dlim, Fast
     reinterpret_cast<ulonglong2 *>(cfg.AC[d & 1])[w] = make_ulonglong2(0, 0);
   unsigned round = 0;
   if (tid == 0) s_seed = level_seed(cfg.seed, d);
-  if (!grid_barrier(&meta->bar, round, &meta->status)) return;
+  if (!grid_barrier(&meta->bar, round, cfg.polls, &meta->status)) return;
   for (;;) {
     const u64 s = s_seed;
     const unsigned m32 = (unsigned)m;
@@ -510,7 +514,7 @@ k_mid(const u64 *__restrict__ keys0, FastMeta *__restrict__ meta, int dlim, Fast
         if ((old[u] >> (p[u] & 31)) & 1ull) atomicOr(AC + (p[u] >> 5), 1ull << (32 + (p[u] & 31)));
     }
     if (tid == 0) s_cnt = s_ones = 0;
-    if (!grid_barrier(&meta->bar, round, &meta->status)) return;
+    if (!grid_barrier(&meta->bar, round, cfg.polls, &meta->status)) return;
     // keep the keys whose bit is not a lone hit; a chunk is read before any of
     // it is written, and what is written lies before what is still to be read
     for (unsigned i0 = 0; i0 < c; i0 += U * kMidThreads) {
@@ -561,7 +565,7 @@ k_mid(const u64 *__restrict__ keys0, FastMeta *__restrict__ meta, int dlim, Fast
       if (s_ones) atomicAdd(&meta->lv[d].weight, (u64)s_ones);
       if (!fits) atomicOr(&meta->status, ST_OVERFLOW);
     }
-    if (!grid_barrier(&meta->bar, round, &meta->status)) return;
+    if (!grid_barrier(&meta->bar, round, cfg.polls, &meta->status)) return;
     if (tid == 0) {
       const u64 nn = __ldcg(&meta->n_out[d]);
       s_nn = nn;
@@ -923,6 +927,7 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
   cfg.Pmax = kPmax;
   cfg.Btarget = (u64)sm_count() * 4;
   cfg.cap_scale = g_cap_scale;
+  cfg.polls = g_mid_polls;
   FastMeta hm;
   memset(&hm, 0, sizeof(hm));
   const u64 m0 = level_bits(N, gamma);
@@ -1125,7 +1130,7 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
     goto fail;
   }
   if (hm.status || !hm.tail_done) {
-    rc = MPHF_EINTERNAL;
+    rc = hm.status & ST_TIMEOUT ? MPHF_ETIMEOUT : MPHF_EINTERNAL;
     goto fail;
   }
   {
@@ -1219,5 +1224,10 @@ extern "C" int mphf_debug_level1_bound(uint64_t N, double gamma, uint64_t btarge
   *capY = bbh::level1_bound(N, gamma, btarget, bbh::kPmax, 1.0, &nh, &bb);
   *n1_hi = nh;
   *Bb = bb;
+  return MPHF_OK;
+}
+
+extern "C" int mphf_debug_mid(int polls) {
+  bbh::g_mid_polls = polls < 0 ? bbh::kMidPolls : (unsigned)polls;
   return MPHF_OK;
 }

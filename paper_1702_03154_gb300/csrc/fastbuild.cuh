@@ -20,7 +20,7 @@ enum : unsigned {
   ST_OVERFLOW = 1u,   // a bucket / buffer bound was exceeded: rebuild with the unbucketed path
   ST_DUPLICATE = 2u,  // equal keys in the fallback
   ST_INTERNAL = 4u,   // a consistency check failed
-  ST_TIMEOUT = 8u
+  ST_TIMEOUT = 8u       // a grid barrier gave up
 };
 
 struct FLevel {
@@ -63,6 +63,7 @@ struct FastCfg {
   u64 T;                // levels with at most T keys run in the single-CTA tail
   u64 Tmid, mmid;       // levels of at most Tmid keys and mmid bits run in k_mid (0: none)
   u64 *AC[2];           // its hit / collision words (mmid / 32 each), by d & 1
+  unsigned polls;       // of its grid barrier before it gives up
   u64 Pmax, Pmin, Btarget;
   double cap_scale;     // bucket capacity multiplier (1 in production; < 1 only in tests)
 };
