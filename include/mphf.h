@@ -187,8 +187,10 @@ int mphf_debug_slabs(uint32_t shift, uint64_t min_ac_bytes);
 
 /* Test hook for the level loop of mid-sized levels (16K to 3.5M keys): looks at
  * its grid barrier before a wait gives up and the build returns MPHF_ETIMEOUT
- * (negative: the default, about a second). */
-int mphf_debug_mid(int polls);
+ * (negative: the default, about a second), and CTAs of its cooperative launch
+ * (0: the default; a launch of more than fit on the device at once is refused,
+ * and those levels then run in buckets). */
+int mphf_debug_mid(int polls, uint32_t ctas);
 
 /* Test hook: scales the bucket capacities of mphf_build_batched (default 1;
  * values < 1 make sets overflow and exercise their individual rebuild). */

@@ -422,6 +422,7 @@ static constexpr u64 kMidBits = 1ull << 24;  // bits of a level at most (4 MB of
 
 static constexpr unsigned kMidPolls = 1u << 22;
 unsigned g_mid_polls = kMidPolls;
+unsigned g_mid_ctas = 0;  // CTAs of a launch (0: one a multiprocessor)
 
 // All CTAs' threads wait here; false after `polls` looks, about a second (the
 // status is raised and the launch winds down).
@@ -894,21 +895,27 @@ static u64 tail_limit(double gamma, u64 *mcap_out) {
 }
 
 // k_mid on levels of at most n keys each, found by the device at levels <= dlim.
-static int launch_mid(const u64 *keys, u64 n, FastMeta *meta, int dlim, const FastCfg &cfg,
-                      cudaStream_t st) {
+// false: the launch was refused (a context that owns fewer multiprocessors than
+// the device reports cannot hold the grid).
+static bool launch_mid(const u64 *keys, u64 n, FastMeta *meta, int dlim, const FastCfg &cfg,
+                       cudaStream_t st) {
   LaunchScope ls("mid", st);
-  const unsigned g = (unsigned)sm_count();
+  const unsigned g = g_mid_ctas ? g_mid_ctas : (unsigned)sm_count();
   void *args[] = {(void *)&keys, (void *)&meta, (void *)&dlim, (void *)&cfg};
-  MPHF_CUDA(cudaLaunchCooperativeKernel((const void *)k_mid, dim3(g), dim3(kMidThreads), args,
-                                        (size_t)ceil_div(n, g) * 8, st));
-  return MPHF_OK;
+  if (cudaLaunchCooperativeKernel((const void *)k_mid, dim3(g), dim3(kMidThreads), args,
+                                  (size_t)ceil_div(n, g) * 8, st) == cudaSuccess)
+    return true;
+  cudaGetLastError();
+  return false;
 }
 
 // Returns MPHF_OK with *fallback_needed = false on success; *fallback_needed =
 // true (and nothing allocated) when a device-side bound was exceeded, or when
-// there is no room for a grouped level's slabs.
-int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaStream_t st,
-               mphf_t *h, bool *fallback_needed, KeyFeed *feed) {
+// there is no room for a grouped level's slabs.  use_mid = false: every level of
+// more than T keys runs in buckets.
+static int fast_build_levels(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed,
+                             cudaStream_t st, mphf_t *h, bool *fallback_needed, KeyFeed *feed,
+                             bool use_mid, bool *refused) {
   *fallback_needed = false;
   int rc = set_attrs();
   if (rc != MPHF_OK) return rc;
@@ -954,7 +961,7 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
   } while (0)
 
   // k_mid's reach (a shrunken bucket capacity, as tests set, keeps to buckets)
-  if (cfg.cap_scale == 1.0) {
+  if (use_mid && cfg.cap_scale == 1.0) {
     cfg.Tmid = std::min(kMidMax, (u64)sm_count() * kMidKeys);
     cfg.mmid = std::min(level_bits(cfg.Tmid, gamma), kMidBits);
     if (cfg.Tmid <= T) cfg.Tmid = 0;
@@ -1004,7 +1011,10 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
     cfg.arena = (u64 *)sc.arena.p;
     if (feed) FTRY(feed->ensure(N, st));
     FCUDA(cudaMemcpyAsync(meta, &hm, sizeof(hm), cudaMemcpyHostToDevice, st));
-    FTRY(launch_mid(keys, N, meta, 0, cfg, st));
+    if (!launch_mid(keys, N, meta, 0, cfg, st)) {
+      *refused = true;
+      goto fail;
+    }
     {
       LaunchScope ls("tail", st);
       k_tail<<<1, kTailThreads, tail_smem_bytes(mcap, T), st>>>(meta, (int)L, cfg, mcap);
@@ -1103,7 +1113,10 @@ int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaS
         k_fill_compact<<<dlim == 0 && hm.lv[0].B < ctas ? (unsigned)hm.lv[0].B : ctas, kTT,
                          fill_smem(dlim == 0 ? hm.lv[0].P : cfg.Pmax), st>>>(meta, dlim, cfg);
       }
-      if (cfg.Tmid) FTRY(launch_mid(nullptr, cfg.Tmid, meta, dlim, cfg, st));
+      if (cfg.Tmid && !launch_mid(nullptr, cfg.Tmid, meta, dlim, cfg, st)) {
+        *refused = true;
+        goto fail;
+      }
       {
         LaunchScope ls("tail", st);
         k_tail<<<1, kTailThreads, tail_smem_bytes(mcap, T), st>>>(meta, cfg.Tmid ? (int)L : dlim,
@@ -1201,6 +1214,15 @@ fail:
 #undef FCUDA
 }
 
+int fast_build(const u64 *keys, u64 N, double gamma, uint32_t L, u64 seed, cudaStream_t st,
+               mphf_t *h, bool *fallback_needed, KeyFeed *feed) {
+  bool refused = false;
+  const int rc = fast_build_levels(keys, N, gamma, L, seed, st, h, fallback_needed, feed, true,
+                                   &refused);
+  if (!refused) return rc;
+  return fast_build_levels(keys, N, gamma, L, seed, st, h, fallback_needed, feed, false, &refused);
+}
+
 }  // namespace bbh
 
 // Test hooks (host arithmetic only, no device work): the bucketed level size
@@ -1227,7 +1249,8 @@ extern "C" int mphf_debug_level1_bound(uint64_t N, double gamma, uint64_t btarge
   return MPHF_OK;
 }
 
-extern "C" int mphf_debug_mid(int polls) {
+extern "C" int mphf_debug_mid(int polls, uint32_t ctas) {
+  bbh::g_mid_ctas = ctas;
   bbh::g_mid_polls = polls < 0 ? bbh::kMidPolls : (unsigned)polls;
   return MPHF_OK;
 }

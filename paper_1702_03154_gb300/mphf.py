@@ -87,7 +87,7 @@ def lib():
         "mphf_batched_debug_config": ([dbl], i32),
         "mphf_debug_slabs": ([u32, u64], i32),
         "mphf_debug_lookup_wide": ([i32], i32),
-        "mphf_debug_mid": ([i32], i32),
+        "mphf_debug_mid": ([i32, u32], i32),
         "mphf_debug_size_level": ([u64, dbl, u64, pu64, pu64, pu64], i32),
         "mphf_debug_level1_bound": ([u64, dbl, u64, pu64, pu64, pu64], i32),
         "mphf_batched_tuning": ([u32, u64, pu64, pu64, pu64], i32),
@@ -474,9 +474,10 @@ def debug_slabs(shift: int = 27, min_ac_bytes: int = 64 << 20) -> None:
     _check(lib().mphf_debug_slabs(int(shift), int(min_ac_bytes)), "mphf_debug_slabs")
 
 
-def debug_mid(polls: int = -1) -> None:
-    """Test hook: polls of the mid-sized levels' grid barrier before it gives up."""
-    _check(lib().mphf_debug_mid(int(polls)), "mphf_debug_mid")
+def debug_mid(polls: int = -1, ctas: int = 0) -> None:
+    """Test hook: polls of the mid-sized levels' grid barrier before it gives up,
+    and the CTAs of their launch."""
+    _check(lib().mphf_debug_mid(int(polls), int(ctas)), "mphf_debug_mid")
 
 
 def batched_tuning(S: int, total_keys: int) -> dict:
