@@ -962,7 +962,7 @@ static int batched_impl(const u64 *d_keys, const u64 *h_off, unsigned S, double 
                         unsigned *n_rebuilt) {
   int rc = MPHF_OK;
   *n_rebuilt = 0;
-  static bool attr = false;
+  static DeviceOnce attrs;
   const size_t split_b = split_smem_bytes((unsigned)kBmax);
   // compaction: per-set destination arrays (Bset_max) + a stage of kTile + kIn
   // + the bucket's slice of A_d; the attribute admits the largest Bset_max
@@ -973,7 +973,7 @@ static int batched_impl(const u64 *d_keys, const u64 *h_off, unsigned S, double 
   while (T > 64 && tail_smem_bytes(level_bits(T, gamma), T, tune.tail_keys) > kBTailSmem) T >>= 1;
   mcap = level_bits(T, gamma);
   const size_t tail_b = tail_smem_bytes(mcap, T, tune.tail_keys);
-  if (!attr) {
+  rc = once_per_device(attrs, [&] {
     MPHF_CUDA(cudaFuncSetAttribute(k_bpartition0<true>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)(split_b + kTile * 8)));
@@ -989,8 +989,9 @@ static int batched_impl(const u64 *d_keys, const u64 *h_off, unsigned S, double 
                                    (int)kBTailSmem));
     MPHF_CUDA(cudaFuncSetAttribute(k_btail<256, 4096>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)kBTailSmem));
-    attr = true;
-  }
+    return (int)MPHF_OK;
+  });
+  if (rc != MPHF_OK) return rc;
   for (unsigned s = 0; s < S; s++) out[s] = nullptr;
   const u64 total = h_off[S] - h_off[0];
   BCfg c;

@@ -554,17 +554,16 @@ static SlabScatterFn slab_scatter_fn(bool al, bool pos, bool one) {
 // slab (p - base) >> shift, nslab slabs; se[i], se[nslab + i] receive slab i's
 // range of out.  slab: 4 * kSlabMax u64 of device scratch.
 static int slab_attrs() {
-  static bool attr = false;
-  if (!attr) {
+  static DeviceOnce attrs;
+  return once_per_device(attrs, [] {
     const int sb = (int)(split_smem_bytes(kSlabMax) + kTile * 8);
     for (int v = 0; v < 8; v++)
       MPHF_CUDA(cudaFuncSetAttribute(slab_scatter_fn(v & 1, v & 2, v & 4),
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, sb));
     MPHF_CUDA(cudaFuncSetAttribute(k_fine_fill, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)kFineSmem));
-    attr = true;
-  }
-  return MPHF_OK;
+    return (int)MPHF_OK;
+  });
 }
 
 // One launch of the slab multisplit: keys F (n) into the ranges cursor[i] ..

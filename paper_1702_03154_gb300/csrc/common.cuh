@@ -134,6 +134,21 @@ inline int sm_count() {
   return cache[dev];
 }
 
+// set() once on each device (a kernel's shared-memory limit belongs to the
+// device that was current when it was set).  Threads that come at the same time
+// may both run it.
+struct DeviceOnce {
+  std::atomic<bool> done[64] = {};
+};
+template <class F>
+inline int once_per_device(DeviceOnce &once, const F &set) {
+  std::atomic<bool> &done = once.done[cur_device()];
+  if (done.load()) return MPHF_OK;
+  const int rc = set();
+  if (rc == MPHF_OK) done.store(true);
+  return rc;
+}
+
 // CTAs of `kernel` (block threads, dynamic smem bytes) that fit on the whole
 // GPU at once: a grid of this size runs in a single wave.
 template <class K>

@@ -664,7 +664,7 @@ k_tail(FastMeta *__restrict__ meta, int dlim, FastCfg cfg, u64 mcap) {
 // ---------------------------------------------------------------------------
 // Host side.
 // ---------------------------------------------------------------------------
-static bool g_attr_set = false;
+static DeviceOnce g_attrs;
 double g_cap_scale = 1.0;
 
 using SplitFn = void (*)(const u64 *, u64, FastMeta *, int, FastCfg, unsigned);
@@ -691,7 +691,6 @@ static FsplitFn fsplit_fn(int nt, bool narrow) {
 }
 
 static int set_attrs() {
-  if (g_attr_set) return MPHF_OK;
   for (int v = 0; v < 4; v++)
     MPHF_CUDA(cudaFuncSetAttribute(split_fn(v & 1 ? kWMaxNb : 1, (v & 2) != 0),
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wc_smem(1)));
@@ -714,7 +713,6 @@ static int set_attrs() {
                                  (int)(kMidKeys * 8)));
   MPHF_CUDA(cudaFuncSetAttribute(k_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kTailSmemMax));
-  g_attr_set = true;
   return MPHF_OK;
 }
 
@@ -917,7 +915,7 @@ static int fast_build_levels(const u64 *keys, u64 N, double gamma, uint32_t L, u
                              cudaStream_t st, mphf_t *h, bool *fallback_needed, KeyFeed *feed,
                              bool use_mid, bool *refused) {
   *fallback_needed = false;
-  int rc = set_attrs();
+  int rc = once_per_device(g_attrs, set_attrs);
   if (rc != MPHF_OK) return rc;
   u64 mcap = 0;
   const u64 T = tail_limit(gamma, &mcap);

@@ -157,17 +157,18 @@ static int split_parts(const u64 *keys, u64 n, uint32_t K, u64 part_seed, DevBuf
   const double mean = (double)n / K;
   *cap = ((u64)(mean + 8.0 * sqrt(mean) + 64.0) + 15) & ~15ull;
   counts.clear();
-  static bool attr = false;
-  if (!attr) {
+  static DeviceOnce attrs;
+  int rc = once_per_device(attrs, [] {
     MPHF_CUDA(cudaFuncSetAttribute(k_part_split<kWT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)wc_smem(1)));
     MPHF_CUDA(cudaFuncSetAttribute(k_part_split<kWT / 2>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wc_smem(2)));
-    attr = true;
-  }
+    return (int)MPHF_OK;
+  });
+  if (rc != MPHF_OK) return rc;
   DevBuf cnt;  // K counts, then the status word
   const size_t words = ((size_t)K + 1) * kCntStride;
-  int rc = dev_alloc(out, K * *cap * sizeof(u64), s);
+  rc = dev_alloc(out, K * *cap * sizeof(u64), s);
   if (rc == MPHF_OK) rc = dev_alloc(cnt, words * sizeof(u64), s);
   std::vector<u64> c(words, 0);
   cudaError_t e = cudaSuccess;
