@@ -414,8 +414,13 @@ __global__ void k_unhash(u64 *__restrict__ F, u64 n, u64 s) {
 // Both sides measured (gamma = 2): build of 2e5 keys 150 us against 225, 1e6 166
 // against 243, 3e6 231 against 330; reach of 1e6 / 3.5e6 keys: build of 3e6 249
 // / 231, of 2e7 strings 1079 / 1061.
+// A CTA takes half a multiprocessor's registers and threads, with eight keys a
+// thread in flight, so that lookups of a server run beside it: with 1024 threads
+// of four keys, builds of 1e5 to 1e6 keys among 1.6e5 requests/s brought the
+// lookups' p99 to 0.091 ms, with 512 to 0.081 (1e6 to 3.4e6: 0.137 / 0.107);
+// builds take the same time (1e6 172 us, 2.7e6 218, 3.4e6 235 / 243).
 // ---------------------------------------------------------------------------
-static constexpr int kMidThreads = 1024;
+static constexpr int kMidThreads = 512;
 static constexpr unsigned kMidKeys = 24576;  // of a CTA
 static constexpr u64 kMidMax = 3500000;      // keys of a level at most
 static constexpr u64 kMidBits = 1ull << 24;  // bits of a level at most (4 MB of words)
@@ -448,7 +453,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &round, uns
   return ok != 0;
 }
 
-__global__ void __launch_bounds__(kMidThreads, 1)
+__global__ void __launch_bounds__(kMidThreads, 2)
 k_mid(const u64 *__restrict__ keys0, FastMeta *__restrict__ meta, int dlim, FastCfg cfg) {
   extern __shared__ __align__(16) unsigned char smem[];
   u64 *keys = reinterpret_cast<u64 *>(smem);
@@ -500,7 +505,7 @@ k_mid(const u64 *__restrict__ keys0, FastMeta *__restrict__ meta, int dlim, Fast
     const unsigned m32 = (unsigned)m;
     u64 *AC = cfg.AC[d & 1];
     auto at = [&](u64 x) { return reduce_range32(mix64(x ^ s), m32); };
-    constexpr unsigned U = 4;
+    constexpr unsigned U = 8;
     for (unsigned i0 = tid; i0 < c; i0 += U * kMidThreads) {
       unsigned p[U];
       u64 old[U];
@@ -899,9 +904,13 @@ static bool launch_mid(const u64 *keys, u64 n, FastMeta *meta, int dlim, const F
                        cudaStream_t st) {
   LaunchScope ls("mid", st);
   const unsigned g = g_mid_ctas ? g_mid_ctas : (unsigned)sm_count();
+  // Past 64 KB of keys a CTA asks for more than half a multiprocessor's shared
+  // memory: two of 106 KB each landed on one (2e6 keys: 122 us, alone 96)
+  size_t smem = (size_t)ceil_div(n, g) * 8;
+  if (smem > 64 * 1024) smem = std::max(smem, (size_t)116 * 1024);
   void *args[] = {(void *)&keys, (void *)&meta, (void *)&dlim, (void *)&cfg};
-  if (cudaLaunchCooperativeKernel((const void *)k_mid, dim3(g), dim3(kMidThreads), args,
-                                  (size_t)ceil_div(n, g) * 8, st) == cudaSuccess)
+  if (cudaLaunchCooperativeKernel((const void *)k_mid, dim3(g), dim3(kMidThreads), args, smem,
+                                  st) == cudaSuccess)
     return true;
   cudaGetLastError();
   return false;
