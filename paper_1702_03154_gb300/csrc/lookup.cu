@@ -64,10 +64,9 @@ static constexpr int kLookupWarps = kLookupThreads / 32;
 // g >> kQShift is below 2^32 (A below 2^36 bits); then a probe's position
 // arithmetic is 32-bit: with off_d a multiple of 64,
 //   g >> kQShift = (off_d >> kQShift) + (p >> kQShift),  g & mask = p & mask.
-// Warp w takes the keys [w csz, (w + 1) csz).
 template <int W, bool kNarrow>
 __global__ void __launch_bounds__(kLookupThreads, W == 15 ? 3 : 4)
-k_lookup(const u64 *__restrict__ keys, u64 n, unsigned csz, u64 *__restrict__ out, LookupArgs a,
+k_lookup(const u64 *__restrict__ keys, RingShape sh, u64 *__restrict__ out, LookupArgs a,
          LevelTable t) {
   using LW = Lay<W>;
   __shared__ u64 ts[MPHF_MAX_LEVELS], tm[MPHF_MAX_LEVELS], toff[MPHF_MAX_LEVELS];
@@ -85,18 +84,17 @@ k_lookup(const u64 *__restrict__ keys, u64 n, unsigned csz, u64 *__restrict__ ou
   const unsigned lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   u64 *ring = rings[threadIdx.x >> 5];
-  const u64 c0 = (((u64)blockIdx.x * kLookupThreads + threadIdx.x) >> 5) * csz;
-  if (c0 >= n) return;
-  const unsigned len = (unsigned)min((u64)csz, n - c0);
-  keys += c0;
-  out += c0;
+  const RingPart mine(sh, (blockIdx.x * kLookupThreads + threadIdx.x) >> 5);
+  const unsigned len = mine.len;
+  if (!len) return;
   unsigned cur = 0;   // keys taken
   unsigned base = 0;  // keys whose indices have left the ring
-  // keys [i0, i0 + 64) of the range into the ring
+  // keys [i0, i0 + 64) of the warp's part into the ring
   auto fetch = [&](unsigned i0) {
+    const u64 *src = keys + mine.place(sh, i0);
 #pragma unroll
-    for (unsigned i = i0 + lane; i < i0 + kBlock; i += 32)
-      if (i < len) key_async(ring + (i & (kRing - 1)), keys + i);
+    for (unsigned u = lane; u < kBlock; u += 32)
+      if (i0 + u < len) key_async(ring + ((i0 + u) & (kRing - 1)), src + u);
     key_commit();
   };
   for (unsigned i = 0; i < min(len, kRing); i += kBlock) fetch(i);
@@ -128,11 +126,12 @@ k_lookup(const u64 *__restrict__ keys, u64 n, unsigned csz, u64 *__restrict__ ou
       const unsigned end = min(base + kBlock, len);
       const bool old = (act[0] && idx[0] < end) || (act[1] && idx[1] < end);
       if (!__any_sync(0xffffffffu, old)) {
+        u64 *dst = out + mine.place(sh, base) + lane;
         __syncwarp();
 #pragma unroll
         for (unsigned u = 0; u < kBlock; u += 32) {
           const unsigned i = base + u + lane;
-          if (i < end) __stcs(out + i, ring[i & (kRing - 1)]);
+          if (i < end) __stcs(dst + u, ring[i & (kRing - 1)]);
         }
         fetch(base + kRing);
         key_wait<1>();
@@ -324,10 +323,10 @@ static int launch_lookup(const u64 *keys, u64 n, u64 *out, const LookupArgs &a,
   static unsigned mb_dev[64] = {0};  // resident CTAs, per device
   unsigned &mb = mb_dev[cur_device()];
   if (!mb) mb = resident_grid(k_lookup<W, NARROW>, kLookupThreads, 0);
-  const unsigned csz = ring_range(n, (u64)mb * kLookupWarps);
-  const u64 grid = ((n + csz - 1) / csz + kLookupWarps - 1) / kLookupWarps;
+  const RingShape sh = ring_shape(n, (u64)mb * kLookupWarps);
   LaunchScope ls("lookup", s);
-  k_lookup<W, NARROW><<<(unsigned)grid, kLookupThreads, 0, s>>>(keys, n, csz, out, a, t);
+  k_lookup<W, NARROW><<<ring_grid(sh, kLookupWarps, mb), kLookupThreads, 0, s>>>(keys, sh, out, a,
+                                                                                 t);
   MPHF_CUDA(cudaGetLastError());
   return MPHF_OK;
 }

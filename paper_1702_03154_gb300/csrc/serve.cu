@@ -301,10 +301,10 @@ k_lookup_multi(const ReqDev *__restrict__ reqs, unsigned nreq, u64 total, u64 cs
 // Lookups against the K functions of a split, without routing the keys: a
 // refilled slot takes its key's part from the part hash, that part's
 // function, and adds the part's offset to the answer.  Slots, probes and the
-// ring as in k_lookup; warp w takes the keys [w csz, (w + 1) csz).
+// ring as in k_lookup.
 template <int W, bool NARROW>
 __global__ void __launch_bounds__(kMultiThreads)
-k_lookup_parts(const u64 *__restrict__ keys, u64 n, unsigned csz, u64 *__restrict__ out,
+k_lookup_parts(const u64 *__restrict__ keys, RingShape sh, u64 *__restrict__ out,
                const LookupDev *const *__restrict__ fns, const u64 *__restrict__ prefix,
                uint32_t K, u64 sp) {
   using LW = Lay<W>;
@@ -312,17 +312,17 @@ k_lookup_parts(const u64 *__restrict__ keys, u64 n, unsigned csz, u64 *__restric
   const unsigned lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   u64 *ring = rings[threadIdx.x >> 5];
-  const u64 c0 = (((u64)blockIdx.x * kMultiThreads + threadIdx.x) >> 5) * csz;
-  if (c0 >= n) return;
-  const unsigned len = (unsigned)min((u64)csz, n - c0);
-  keys += c0;
-  out += c0;
+  const RingPart mine(sh, (blockIdx.x * kMultiThreads + threadIdx.x) >> 5);
+  const unsigned len = mine.len;
+  if (!len) return;
   unsigned cur = 0;   // keys taken
   unsigned base = 0;  // keys whose indices have left the ring
+  // keys [i0, i0 + 64) of the warp's part into the ring
   auto fetch = [&](unsigned i0) {
+    const u64 *src = keys + mine.place(sh, i0);
 #pragma unroll
-    for (unsigned i = i0 + lane; i < i0 + kBlock; i += 32)
-      if (i < len) key_async(ring + (i & (kRing - 1)), keys + i);
+    for (unsigned u = lane; u < kBlock; u += 32)
+      if (i0 + u < len) key_async(ring + ((i0 + u) & (kRing - 1)), src + u);
     key_commit();
   };
   for (unsigned i = 0; i < min(len, kRing); i += kBlock) fetch(i);
@@ -365,11 +365,12 @@ k_lookup_parts(const u64 *__restrict__ keys, u64 n, unsigned csz, u64 *__restric
 #pragma unroll
       for (int s = 0; s < kMultiSlots; s++) old |= act[s] && idx[s] < end;
       if (!__any_sync(0xffffffffu, old)) {
+        u64 *dst = out + mine.place(sh, base) + lane;
         __syncwarp();
 #pragma unroll
         for (unsigned u = 0; u < kBlock; u += 32) {
           const unsigned i = base + u + lane;
-          if (i < end) __stcs(out + i, ring[i & (kRing - 1)]);
+          if (i < end) __stcs(dst + u, ring[i & (kRing - 1)]);
         }
         fetch(base + kRing);
         key_wait<1>();
@@ -424,11 +425,10 @@ static int launch_parts_wn(const LookupDev *const *d_fns, const u64 *prefix, uin
   static u64 maxb_dev[64] = {0};  // one wave of resident CTAs, per device
   u64 &maxb = maxb_dev[cur_device()];
   if (!maxb) maxb = resident_grid(k_lookup_parts<W, NARROW>, kMultiThreads, 0);
-  const unsigned csz = ring_range(n, maxb * (kMultiThreads / 32));
-  const u64 grid = ((n + csz - 1) / csz + (kMultiThreads / 32) - 1) / (kMultiThreads / 32);
+  const RingShape sh = ring_shape(n, maxb * (kMultiThreads / 32));
   LaunchScope ls("lookup_parts", s);
-  k_lookup_parts<W, NARROW><<<(unsigned)grid, kMultiThreads, 0, s>>>(keys, n, csz, out, d_fns,
-                                                                      prefix, K, sp);
+  k_lookup_parts<W, NARROW><<<ring_grid(sh, kMultiThreads / 32, maxb), kMultiThreads, 0, s>>>(
+      keys, sh, out, d_fns, prefix, K, sp);
   MPHF_CUDA(cudaGetLastError());
   return MPHF_OK;
 }
