@@ -173,16 +173,23 @@ k_lookup(const u64 *__restrict__ keys, RingShape sh, u64 *__restrict__ out, Look
   }
 }
 
-// 8-byte units: each slot loads its next key itself and stores its index when
-// its key retires (no ring).  Their probes are ordinary cached loads that lean
-// on a large L1 for the requests in flight, and the rings' 128 KB of shared
-// memory a multiprocessor leave little of it: 1e8 queries of a function in L2
-// 1.01 ms, 1.52 with the ring.  Warps take chunks of csz keys in a fixed order.
-template <bool kNarrow>
+// Without a ring: each slot loads its next key itself and stores its index when
+// its key retires; warps take chunks of csz keys in a fixed order.  For
+//  - 8-byte units: their probes are ordinary cached loads that lean on a large L1
+//    for the requests in flight, and the rings' 128 KB of shared memory a
+//    multiprocessor leave little of it: 1e8 queries of a function in L2 1.01 ms,
+//    1.52 with the ring;
+//  - 32-byte sectors where a warp has 128 to 1024 keys: the ring's first 512 keys
+//    would arrive before the first probe, and it leaves block by block at the end.
+//    8e5 queries of a 3e7-key function 21.0 us (22.8 with the ring), 2.5e6 40.3
+//    (42.0), 3e6 at gamma 5 34.2 (36.0), with 5% absent keys 44.3 (50.4); below
+//    and above that range the ring is as fast or faster (5e5 18.7 / 18.6, 6e6
+//    77.1 / 76.4 us).
+template <int W, bool kNarrow>
 __global__ void __launch_bounds__(kLookupThreads)
-k_lookup_units(const u64 *__restrict__ keys, u64 n, u64 csz, u64 *__restrict__ out, LookupArgs a,
-               LevelTable t) {
-  using LW = Lay<(int)kUnitBits>;
+k_lookup_direct(const u64 *__restrict__ keys, u64 n, u64 csz, u64 *__restrict__ out, LookupArgs a,
+                LevelTable t) {
+  using LW = Lay<W>;
   __shared__ u64 ts[MPHF_MAX_LEVELS], tm[MPHF_MAX_LEVELS], toff[MPHF_MAX_LEVELS];
   __shared__ unsigned tm32[MPHF_MAX_LEVELS], toq[MPHF_MAX_LEVELS];
   for (unsigned i = threadIdx.x; i < a.L_used; i += kLookupThreads) {
@@ -272,8 +279,8 @@ k_lookup_units(const u64 *__restrict__ keys, u64 n, u64 csz, u64 *__restrict__ o
     if (!__any_sync(0xffffffffu, any)) break;
 
     // one probe per active slot: issue all loads, then resolve
-    LW::Pos p[2];
-    LW::Data v[2];
+    typename LW::Pos p[2];
+    typename LW::Data v[2];
 #pragma unroll
     for (int s = 0; s < 2; s++) {
       if (act[s]) {
@@ -331,21 +338,31 @@ static int launch_lookup(const u64 *keys, u64 n, u64 *out, const LookupArgs &a,
   return MPHF_OK;
 }
 
-template <bool NARROW>
-static int launch_lookup_units(const u64 *keys, u64 n, u64 *out, const LookupArgs &a,
-                               const LevelTable &t, cudaStream_t s) {
+template <int W, bool NARROW>
+static int launch_lookup_direct(const u64 *keys, u64 n, u64 *out, const LookupArgs &a,
+                                const LevelTable &t, cudaStream_t s) {
   // one wave of resident CTAs: a second would only start after the first has
   // drained
   static unsigned mb_dev[64] = {0};  // per device
   unsigned &mb = mb_dev[cur_device()];
-  if (!mb) mb = resident_grid(k_lookup_units<NARROW>, kLookupThreads, 0);
-  const u64 csz = lookup_chunk(n, (u64)mb * kLookupWarps);
+  if (!mb) mb = resident_grid(k_lookup_direct<W, NARROW>, kLookupThreads, 0);
+  const u64 warps = (u64)mb * kLookupWarps;
+  // sectors: two chunks a warp, so that a stretch of deep keys does not fall to
+  // a few warps alone (3e6 queries, the first tenth absent: 50.6 us, 62.1 in one)
+  const u64 csz = W == (int)kUnitBits ? lookup_chunk(n, warps)
+                                      : ((n + 2 * warps - 1) / (2 * warps) + 15) & ~15ull;
   const u64 grid = ((n + csz - 1) / csz + kLookupWarps - 1) / kLookupWarps;
   LaunchScope ls("lookup", s);
-  k_lookup_units<NARROW><<<(unsigned)(grid > mb ? mb : grid), kLookupThreads, 0, s>>>(
+  k_lookup_direct<W, NARROW><<<(unsigned)(grid > mb ? mb : grid), kLookupThreads, 0, s>>>(
       keys, n, csz, out, a, t);
   MPHF_CUDA(cudaGetLastError());
   return MPHF_OK;
+}
+
+// A batch of 32-byte sector lookups that is better without the ring.
+static bool better_direct(u64 n) {
+  const u64 warps = (u64)sm_count() * 4 * kLookupWarps;
+  return n > 128 * warps && n <= 1024 * warps;
 }
 
 int lookup_impl(const mphf_t *h, const u64 *keys, u64 n, u64 *out, cudaStream_t s) {
@@ -357,8 +374,11 @@ int lookup_impl(const mphf_t *h, const u64 *keys, u64 n, u64 *out, cudaStream_t 
     return narrow ? launch_lookup<kSectWordsMini, true>(keys, n, out, a, t, s)
                   : launch_lookup<kSectWordsMini, false>(keys, n, out, a, t, s);
   if (h->sw == kUnitBits)
-    return narrow ? launch_lookup_units<true>(keys, n, out, a, t, s)
-                  : launch_lookup_units<false>(keys, n, out, a, t, s);
+    return narrow ? launch_lookup_direct<(int)kUnitBits, true>(keys, n, out, a, t, s)
+                  : launch_lookup_direct<(int)kUnitBits, false>(keys, n, out, a, t, s);
+  if (better_direct(n))
+    return narrow ? launch_lookup_direct<kSectWords, true>(keys, n, out, a, t, s)
+                  : launch_lookup_direct<kSectWords, false>(keys, n, out, a, t, s);
   return narrow ? launch_lookup<kSectWords, true>(keys, n, out, a, t, s)
                 : launch_lookup<kSectWords, false>(keys, n, out, a, t, s);
 }
