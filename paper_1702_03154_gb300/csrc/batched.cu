@@ -706,7 +706,12 @@ __global__ void __launch_bounds__(kTT, 2) k_bcompact(int d, BCfg c) {
 // threads with ~MAXK * 8 bytes of shared memory, so that several tails share
 // an SM (the tail is a chain of short, barrier-bound levels).  Two shapes are
 // compiled; the autotuner picks one per size class.
-static constexpr size_t kBTailSmem = 112 * 1024;  // two CTAs a multiprocessor
+// Shared memory of a tail at most, without its positions and with them: two CTAs
+// share a multiprocessor up to gamma 8, one has it from there to gamma 16 (2000
+// sets of 4100 to 8192 keys at gamma 10: levels 0.20 ms; with tails of half the
+// keys, so that still two fit, 0.87).
+static constexpr size_t kBTailBits = 96 * 1024;
+static constexpr size_t kBTailSmem = kBTailBits + 8192 * 4;
 
 template <int NT, int MAXK>
 __global__ void __launch_bounds__(NT) k_btail(BCfg c, u64 mcap, int dlim) {
@@ -970,7 +975,7 @@ static int batched_impl(const u64 *d_keys, const u64 *h_off, unsigned S, double 
   const size_t comp_max = split_smem_bytes((unsigned)kBmax, kTile + kIn) + kPmax / 8;
   u64 mcap = 0;
   u64 T = tune.tail_keys;  // keep a tail's shared memory small enough for several CTAs per SM
-  while (T > 64 && tail_smem_bytes(level_bits(T, gamma), T, tune.tail_keys) > kBTailSmem) T >>= 1;
+  while (T > 64 && tail_smem_bytes(level_bits(T, gamma), 0, tune.tail_keys) > kBTailBits) T >>= 1;
   mcap = level_bits(T, gamma);
   const size_t tail_b = tail_smem_bytes(mcap, T, tune.tail_keys);
   rc = once_per_device(attrs, [&] {
