@@ -741,7 +741,7 @@ __global__ void __launch_bounds__(NT) k_btail(BCfg c, u64 mcap, int dlim) {
   }
   TailSmem sm = carve_tail(smem, mcap, c.T, MAXK);
   const u64 *src = st->small ? c.keys + st->key_off : c.flat + st->flat_off;
-  stage_keys<NT, MAXK>(src, (unsigned)n, sm.keys, [](u64 v) { return v; });
+  stage_keys<NT>(src, (unsigned)n, sm.keys, [](u64 v) { return v; });
   if (threadIdx.x == 0) {
     hist[st->small ? 0 : t].n = n;
     hist[st->small ? 0 : t].off = off;

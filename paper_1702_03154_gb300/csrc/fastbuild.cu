@@ -320,8 +320,8 @@ k_fill_compact(FastMeta *__restrict__ meta, int d, FastCfg cfg) {
 // then, a batch of slabs at a time, each slab's values to its fine buckets of
 // 2^kGroupShift positions (k_fsplit: a group of CTAs per slab) and the batch's
 // buckets filled and compacted (k_gfill).  Measured at 3e9 keys (gamma = 2):
-// coarse 20.4 ms, fine 19.5, fill and compaction 15.7 for the three grouped
-// levels (4.6e9 values, 16 bytes a split), build 60 ms; counting-sort
+// coarse 20.5 ms, fine 18.8, fill and compaction 14.6 for the three grouped
+// levels (4.6e9 values, 16 bytes a split), build 58 ms; counting-sort
 // multisplits and a fill from stored positions took 54.5 + 23.1 ms, build 81.
 // ---------------------------------------------------------------------------
 static constexpr unsigned kGroupShift = 17;
@@ -481,10 +481,10 @@ k_mid(const u64 *__restrict__ keys0, FastMeta *__restrict__ meta, int dlim, Fast
   const u64 lo = min(n, per * blockIdx.x);
   unsigned c = (unsigned)min(per, n - lo);  // this CTA's keys
   if (d == 0) {
-    stage_keys<kMidThreads, (int)kMidKeys>(keys0 + lo, c, keys, [](u64 v) { return v; });
+    stage_keys<kMidThreads>(keys0 + lo, c, keys, [](u64 v) { return v; });
   } else {
     const u64 s_b = level_seed(cfg.seed, d - 1);
-    stage_keys<kMidThreads, (int)kMidKeys>(cfg.F + lo, c, keys,
+    stage_keys<kMidThreads>(cfg.F + lo, c, keys,
                                            [=](u64 v) { return unmix64(v) ^ s_b; });
   }
   // words [w0, w1) of a level are this CTA's to clear and to write out
@@ -608,12 +608,9 @@ k_mid(const u64 *__restrict__ keys0, FastMeta *__restrict__ meta, int dlim, Fast
 }
 
 // ---------------------------------------------------------------------------
-// Single-CTA level loop: levels d0.. of a key set of at most kTailMaxKeys keys,
-// keys and bit arrays in shared memory.  Writes A_d words, level metadata and
-// the sorted fallback.
-// ---------------------------------------------------------------------------
 // Tail of the bucketed build: finds the first level (<= dlim) whose keys were
-// sent to the flat buffer and runs the remaining levels there.
+// sent to the flat buffer and runs the remaining levels there (cta_levels).
+// ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kTailThreads, 1)
 k_tail(FastMeta *__restrict__ meta, int dlim, FastCfg cfg, u64 mcap) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -653,7 +650,7 @@ k_tail(FastMeta *__restrict__ meta, int dlim, FastCfg cfg, u64 mcap) {
   TailSmem sm = carve_tail(smem, mcap, cfg.T);
   // F holds the values of the level before (at t = 0 the caller's keys)
   const u64 s_b = t > 0 ? level_seed(cfg.seed, t - 1) : 0;
-  stage_keys<kTailThreads, (int)kTailMaxKeys>(
+  stage_keys<kTailThreads>(
       cfg.F, (unsigned)n, sm.keys, [=](u64 v) { return t > 0 ? unmix64(v) ^ s_b : v; });
   __syncthreads();
   unsigned used = cta_levels<kTailThreads, (int)kTailMaxKeys>(

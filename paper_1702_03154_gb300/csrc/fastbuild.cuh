@@ -422,7 +422,7 @@ static __device__ void bitonic_sort_smem(u64 *a, unsigned n) {
 
 // dst[i] = f(src[i]), i < n: eight loads of a thread in flight (one at a time,
 // their latency was a third of a 10007-key tail).
-template <int NT, int MAXK, class F>
+template <int NT, class F>
 static __device__ __forceinline__ void stage_keys(const u64 *__restrict__ src, unsigned n,
                                                   u64 *__restrict__ dst, const F &f) {
 #pragma unroll 1

@@ -18,10 +18,11 @@
 // So nothing else may wait or scatter: a warp's keys arrive in a ring in shared
 // memory by asynchronous copies ahead of the slots, the indices replace them
 // there and leave in input order, a block of 64 at a time, once every key of
-// the block has retired.  Measured: 1e8 queries of a 2e9-key function 3.63 ms
-// (3.94 with each key loaded when its slot is refilled and each index stored
-// when its key retires), 2.3e7 queries at gamma 1 in 64-byte sectors 0.57 ms
-// (0.67), 1e8 queries of a function in L2 1.03 ms (1.03).
+// the block has retired.  Measured, with the ring and with each key loaded when
+// its slot is refilled and each index stored when its key retires: 1e8 queries of
+// a 2e9-key function 3.64 / 3.70 ms, of a function in L2 1.03 / 1.06, with a
+// tenth of absent keys 1.21 / 1.14 (a deep key holds its block back), 3e7 queries
+// at gamma 1 0.49 / 0.55, in 64-byte sectors 0.72 / 0.83.
 #include <cuda_runtime.h>
 #include <stdlib.h>
 
