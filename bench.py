@@ -420,22 +420,22 @@ def kernel_table(h, prof, steps, n_queries):
 # the kernel and traffic is null.  Units: a "grouped key" is one key of a level
 # grouped in two splits; a "query" one looked-up key.
 _HDR = ["common.cuh", "fastbuild.cuh", "sector.cuh"]
-_GROUPED = {"src": ["fastbuild.cu", "split.cuh"] + _HDR, "sha": "2e064e8e4923", "unit": "grouped key"}
-_LOOKUP = {"src": ["lookup.cu", "keyring.cuh"] + _HDR, "sha": "cbb66b001393", "unit": "query"}
+_GROUPED = {"src": ["fastbuild.cu", "split.cuh"] + _HDR, "sha": "e85a0725f1ea", "unit": "grouped key"}
+_LOOKUP = {"src": ["lookup.cu", "keyring.cuh"] + _HDR, "sha": "475a48d0c3a0", "unit": "query"}
 NCU_TRAFFIC = {
     "split_coarse": {**_GROUPED, "bytes_per_unit": 15.85,
                      "note": "4e8-key builds (level 0 grouped: 4 launches, 25.36 GB over 1.6e9 "
                              "grouped keys)"},
     "split_fine": {**_GROUPED, "bytes_per_unit": 15.54,
-                   "note": "4e8-key builds (12 launches, 24.87 GB over 1.6e9 grouped keys)"},
+                   "note": "4e8-key builds (12 launches, 24.86 GB over 1.6e9 grouped keys)"},
     "fill_grouped": {**_GROUPED, "bytes_per_unit": 15.64,
                      "note": "4e8-key builds (12 launches, 25.03 GB over 1.6e9 grouped keys)"},
-    "lookup@hbm": {**_LOOKUP, "bytes_per_unit": 136.4,
+    "lookup@hbm": {**_LOOKUP, "bytes_per_unit": 136.3,
                    "note": "4e8-key function (A 188 MB, above L2), 3e7 random member queries x 4 "
-                           "launches, 16.37 GB"},
-    "lookup@l2": {**_LOOKUP, "bytes_per_unit": 14.91,
+                           "launches, 16.35 GB"},
+    "lookup@l2": {**_LOOKUP, "bytes_per_unit": 14.88,
                   "note": "3e7-key function (A 14 MB, in L2), 3e7 random member queries x 4 "
-                          "launches, 1.789 GB"},
+                          "launches, 1.786 GB"},
 }
 L2_BYTES = 126 << 20
 
